@@ -191,6 +191,7 @@ struct hr_work {
     unsigned max_intervals;
     unsigned max_jobs;
     unsigned tile;                   // records per work item (set per kernel variant)
+    unsigned clear_words;            // shadow words per clear item (likewise)
     unsigned consumers;              // per-warp completions per work item
     unsigned cas_cap;                // CAS retries before HR_ERR_CONTENTION
     unsigned long long wait_ns;      // bound of every device-side wait
@@ -270,6 +271,16 @@ constexpr unsigned hr_variant_tile(unsigned v)
            : v == HR_BIN_VARIANT       ? hr_variant_tile(HR_BIN_FALLBACK)
                                        : HR_VARIANTS[v].consumers * 32u * HR_VARIANTS[v].rpl;
 }
+// hr_runs.cu: which checks of one trace it takes, and its work items (one step of
+// a warp).  The others run hr_check_kernel: batches, and the shapes of variants 4
+// and 5 (hr_runs.cu says what each is better at).
+constexpr unsigned HR_RUN_EVERY_RPL = 4;  // records per lane in every-epoch regions
+constexpr bool hr_variant_runs(unsigned v) { return v < 4 || v == HR_EVERY_EPOCH_VARIANT; }
+constexpr unsigned hr_run_tile(unsigned v)
+{
+    return 32u * (v == HR_EVERY_EPOCH_VARIANT ? HR_RUN_EVERY_RPL : (unsigned)HR_VARIANTS[v].rpl);
+}
+constexpr unsigned HR_RUN_CLEAR_WORDS = 1u << 13;  // shadow words per clear item
 #ifndef HR_RING_DEPTH
 #define HR_RING_DEPTH 2
 #endif
@@ -297,6 +308,9 @@ constexpr unsigned long long HR_KEY_MASK = 0xFFFFFFFFFFFFull;
 cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w, const hr_jobd* jobs, unsigned n_jobs,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream,
                            cudaEvent_t before_check, unsigned* launches = nullptr);
+// the per-wave checker of a single trace of n records (hr_variant_runs(variant)), after the pre-pass (hr_runs.cu)
+cudaError_t hr_launch_runs(hr_region_dev* d_regions, const hr_work& w, unsigned long long n,
+                           const unsigned char* d_table, unsigned variant, cudaStream_t stream);
 // interval size and count for a job of n records when it may use up to budget intervals
 void hr_plan_intervals(unsigned long long n, unsigned budget, unsigned* G, unsigned* n_int);
 int hr_check_grid_size(unsigned variant);

@@ -23,7 +23,7 @@
 // of Algorithm 1 (hr_fsm_step) and a 64-bit atomicCAS on its shadow word.
 #include <cuda_runtime.h>
 
-#include "hr_internal.h"
+#include "hr_check.cuh"
 
 namespace {
 
@@ -40,20 +40,6 @@ __device__ __forceinline__ unsigned long long key_at(const hr_record* t, unsigne
 {
     const unsigned long long* p = reinterpret_cast<const unsigned long long*>(t + i) + 1;
     return (__ldg(p) & HR_KEY_MASK) + kb;
-}
-
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p)
-{
-    unsigned v;
-    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-    return v;
-}
-
-__device__ __forceinline__ unsigned long long globaltimer()
-{
-    unsigned long long t;
-    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
-    return t;
 }
 
 // job holding global pre-pass interval i (jobs sorted by int_begin)
@@ -250,7 +236,7 @@ __device__ __forceinline__ void wave_plan(const hr_work& w, const hr_jobd& jb, c
     const unsigned long long end = L + 1 < jb.n_waves ? w.wave_start[g + 1] : jb.n;
     w.wave_end[g] = end;
     *rec_items = (unsigned)((end - w.wave_start[g] + w.tile - 1) / w.tile);
-    *clr_items = *clear ? (unsigned)((rg.n_words + HR_CLEAR_WORDS - 1) / HR_CLEAR_WORDS) : 0u;
+    *clr_items = *clear ? (unsigned)((rg.n_words + w.clear_words - 1) / w.clear_words) : 0u;
 }
 
 // One job: stages follow its waves; threads take waves in parallel.
@@ -593,18 +579,6 @@ __device__ __forceinline__ unsigned smem_add_acq_rel(unsigned* p, unsigned v)
     return old;
 }
 
-__device__ __forceinline__ unsigned atom_add_release(unsigned* p, unsigned v)
-{
-    unsigned old;
-    asm volatile("atom.release.gpu.global.add.u32 %0, [%1], %2;" : "=r"(old) : "l"(p), "r"(v) : "memory");
-    return old;
-}
-
-__device__ __forceinline__ void red_release_add(unsigned* p, unsigned v)
-{
-    asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 // Bounded mbarrier wait: gives up (and raises the abort flag) after wait_ns
 // or when another CTA aborted.
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, unsigned* abort_flag, unsigned* err,
@@ -718,102 +692,6 @@ __device__ __forceinline__ Retry retry_cas(unsigned long long* shadow, unsigned 
         }
     }
     return r;
-}
-
-// Every-epoch mode for a lane's RPL accesses at once (bit k of `act`: slot k
-// holds one): the steps of hr_ep_apply, each over every slot before the next,
-// so each step costs one round trip for all of them and one fence serves them
-// all.  Per access: fold it into the summaries of the conflict kinds it holds
-// (CAS loops), then a sequentially consistent fence, then read the summaries
-// of the kinds it conflicts with; a conflicting holder is reported once per
-// (word, kernel, epoch) through a CAS on the stamp word.  Of two concurrent
-// conflicting accesses at least one therefore sees the other.  Returns 0 or
-// HR_ERR_CONTENTION when a CAS loop reached `cap` tries.
-template <int RPL>
-__device__ __forceinline__ unsigned every_epoch_slots(unsigned long long* shadow, unsigned long long n_words,
-                                                      unsigned act, const unsigned* idx, const unsigned* report_word,
-                                                      const unsigned* tid, const unsigned* op, unsigned bc,
-                                                      unsigned wc, unsigned kernel, const hr_geom& g,
-                                                      hr_region_dev* region, unsigned cap)
-{
-    const unsigned ktag = kernel & 7u;
-    unsigned err = 0;
-    auto holds = [&](int k) { return op[k] == HR_R ? 1u : (op[k] == HR_A ? 2u : 3u); };
-    auto against = [&](int k) { return op[k] == HR_R ? 2u : (op[k] == HR_A ? 1u : 3u); };
-    // 1. the held kinds' summaries, all loaded at once, then every first CAS
-    unsigned long long o[RPL][2], seen[RPL][2];
-    unsigned casm = 0;  // bit 2k+b: a CAS went out on summary b of slot k
-#pragma unroll
-    for (int k = 0; k < RPL; ++k)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-            if (((act >> k) & 1u) && ((holds(k) >> b) & 1u)) o[k][b] = hr_ld_relaxed(shadow + b * n_words + idx[k]);
-#pragma unroll
-    for (int k = 0; k < RPL; ++k)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            if (!((act >> k) & 1u) || !((holds(k) >> b) & 1u)) continue;
-            const unsigned long long n = hr_ep_update(o[k][b], tid[k], bc, wc, ktag, g);
-            if (n == o[k][b]) continue;
-            seen[k][b] = atomicCAS(shadow + b * n_words + idx[k], o[k][b], n);
-            casm |= 1u << (2 * k + b);
-        }
-    // a CAS that lost: fold again into what it saw
-#pragma unroll
-    for (int k = 0; k < RPL; ++k)
-#pragma unroll
-        for (int b = 0; b < 2; ++b) {
-            if (!((casm >> (2 * k + b)) & 1u) || seen[k][b] == o[k][b]) continue;
-            unsigned long long* p = shadow + b * n_words + idx[k];
-            unsigned long long cur = seen[k][b];
-            bool ok = false;
-            for (unsigned tries = 1; tries < cap; ++tries) {
-                const unsigned long long n = hr_ep_update(cur, tid[k], bc, wc, ktag, g);
-                if (n == cur) { ok = true; break; }
-                const unsigned long long sv = atomicCAS(p, cur, n);
-                if (sv == cur) { ok = true; break; }
-                cur = sv;
-            }
-            if (!ok) {
-                err = HR_ERR_CONTENTION;
-                act &= ~(1u << k);  // this access is not applied: it reports nothing
-            }
-        }
-    if (!act) return err;
-    asm volatile("fence.sc.gpu;" ::: "memory");
-    // 2. the conflicting kinds' summaries, all loaded at once
-    unsigned long long sv[RPL][2];
-#pragma unroll
-    for (int k = 0; k < RPL; ++k)
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-            if (((act >> k) & 1u) && ((against(k) >> b) & 1u)) sv[k][b] = hr_ld_relaxed(shadow + b * n_words + idx[k]);
-    // 3. a conflicting holder: claim the (kernel, epoch) of the report
-#pragma unroll
-    for (int k = 0; k < RPL; ++k) {
-        if (!((act >> k) & 1u)) continue;
-        unsigned prior = 0;
-#pragma unroll
-        for (int b = 0; b < 2; ++b)
-            if (!prior && ((against(k) >> b) & 1u) && hr_ep_pred(sv[k][b], tid[k], bc, wc, ktag, g))
-                prior = hr_ep_level(sv[k][b], ktag);
-        if (!prior) continue;
-        unsigned long long* st = shadow + 2 * n_words + idx[k];
-        const unsigned long long mine = ((((unsigned long long)kernel) << 16) | bc) + 1ull;
-        unsigned long long cur = hr_ld_relaxed(st);
-        bool claimed = false;
-        for (unsigned tries = 0; cur < mine && tries < cap; ++tries) {
-            const unsigned long long x = atomicCAS(st, cur, mine);
-            if (x == cur) { claimed = true; break; }
-            cur = x;
-        }
-        if (claimed)
-            hr_append_race(region->ring, region->ring_cap, &region->n_races, &region->flags, report_word[k], tid[k],
-                           kernel, bc, region->region, op[k], prior);
-        else if (cur < mine)
-            err = HR_ERR_CONTENTION;
-    }
-    return err;
 }
 
 template <int TILE>
@@ -1344,9 +1222,10 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
     if (binned && (n_jobs != 1 || !w_in.bin.table)) return cudaErrorInvalidValue;
     if (binned) variant = HR_BIN_FALLBACK;  // the per-wave checker runs after it (and finds no work when binned)
     hr_work w = w_in;
-    w.tile = hr_variant_tile(variant);
+    const bool runs = n_jobs == 1 && hr_variant_runs(variant);
+    w.tile = runs ? hr_run_tile(variant) : hr_variant_tile(variant);
+    w.clear_words = runs ? HR_RUN_CLEAR_WORDS : HR_CLEAR_WORDS;
     w.consumers = hr_variant_consumers(variant);
-    const int grid = hr_check_grid_size(variant);
     if (n_jobs == 0 || n_jobs > HR_MAX_BATCH || n_jobs > w.max_jobs) return cudaErrorInvalidValue;
     const unsigned total_int = jobs[n_jobs - 1].int_begin + jobs[n_jobs - 1].n_int;
     if (total_int > w.max_intervals) return cudaErrorInvalidValue;
@@ -1373,6 +1252,8 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
         const cudaError_t e = hr_launch_binned(d_regions, w, d_table, stream);
         if (e != cudaSuccess) return e;
     }
+    if (runs) return hr_launch_runs(d_regions, w, jobs[0].n, d_table, variant, stream);
+    const int grid = hr_check_grid_size(variant);
     switch (variant) {
     case 0: launch_variant<true, 4, 8>(grid, d_regions, w, d_table, stream); break;
     case 1: launch_variant<false, 4, 8>(grid, d_regions, w, d_table, stream); break;
