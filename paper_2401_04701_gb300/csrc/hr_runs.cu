@@ -28,9 +28,8 @@
 //     rate while the average slice is at 11 %.
 //
 // Measured on the power-law push (2^22 vertices, 537M records, 4 waves): 9.95 ms
-// with hr_check_kernel's best shape, 4.9 ms here (variant 3; 92 G accesses/s at
-// 2.6 TB/s of records: limited by the latency of the loads and CASes, 40 % issue
-// active).  Short waves are bound by the hand-over from stage to stage, which
+// with hr_check_kernel's best shape, 4.53 ms here (variant 3; 118 G accesses/s at
+// 1.9 TB/s of records: limited by the latency of the loads and CASes).  Short waves are bound by the hand-over from stage to stage, which
 // hr_check_kernel's tiles, claimed and copied ahead by a producer warp, do better:
 // batches of many traces (64 uneven traces: 2.4 ms there, 2.7 ms here) and variants
 // 4 and 5 stay with it (tree reduction, 1.03M records in 8 waves: 87 us there,
@@ -45,6 +44,7 @@ constexpr int CONS = 8;                        // warps per CTA
 constexpr int CHECK_THREADS = CONS * 32;
 constexpr unsigned KNOWN = 64;                 // slots of the CTA's table of finished stages
 constexpr unsigned SEEN = 2048;                // entries of the CTA's table of absorbed accesses
+constexpr unsigned FLIGHT = 1024;              // entries of the CTA's table of accesses being CASed
 constexpr unsigned MAX_CLAIM = 16;             // items a warp claims at a time, at most
 
 // What a warp keeps of its current stage and region, in shared memory: it is
@@ -126,6 +126,16 @@ __device__ __forceinline__ bool stage_wait(const unsigned* done, unsigned need, 
 // absorbs everything, until the kernel ends).  A later access of that kind skips
 // its shadow load: without that, the words all threads touch keep one L2 slice
 // busy while the others idle.  64-bit entries, written and read whole.
+//
+// Until such a state is seen, a stage's first accesses of a hub word all CAS it: a
+// quarter of a 1.3M-record stage is in flight at once, and CASes of one word pass
+// one after the other.  A table of the accesses (word, op) the CTA has a CAS out
+// for lets one of them go; the others load the word again afterwards and mostly
+// find themselves absorbed.  Power-law pushes, variants 0 and 3, without and with it:
+// 40,000 vertices (2.56M records, 2 waves) 194 and 290 us, 157 and 160 us; 2^22
+// vertices 5.49 and 4.83 ms (variants 1 and 3), 5.47 and 4.53 ms.
+__device__ __forceinline__ unsigned flight_key(unsigned word, unsigned op) { return ((word << 2) | op) + 1u; }
+__device__ __forceinline__ unsigned flight_slot(unsigned word) { return word % FLIGHT; }
 __device__ __forceinline__ unsigned seen_slot(unsigned word) { return word % SEEN; }
 __device__ __forceinline__ unsigned long long seen_key(unsigned word, unsigned stamp)
 {
@@ -212,6 +222,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
     __shared__ Queue<EVERY ? 1 : QCAP> s_queue[EVERY ? 1 : CONS];
     __shared__ unsigned s_known[KNOWN];
     __shared__ unsigned long long s_seen[EVERY ? 1 : SEEN];
+    __shared__ unsigned s_flight[EVERY ? 1 : FLIGHT];  // flight_key() of an access, or 0
     __shared__ unsigned s_first;
 
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -229,6 +240,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
     if (!EVERY) {
         for (unsigned i = threadIdx.x; i < SEEN; i += CHECK_THREADS) s_seen[i] = ~0ull;
         for (unsigned i = threadIdx.x; i < 2048; i += CHECK_THREADS) s_abs[i] = (unsigned char)absorbs(gtable, i);
+        for (unsigned i = threadIdx.x; i < FLIGHT; i += CHECK_THREADS) s_flight[i] = 0u;
     }
     WarpItem& it = s_item[wid];
     if (lane == 0) {
@@ -399,6 +411,8 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
             queued -= n;
             unsigned long long seen[RPL];
             unsigned casm = 0;   // bit k: a CAS went out for slot k
+            unsigned defer = 0;  // bit k: the CTA has a CAS out for this access already
+            unsigned own = 0;    // bit k: slot k's CAS is entered in the table of those
             unsigned race = 0;   // a byte per slot: 0, or 1 + the prior state of a word this fold moves into RACE
             unsigned whose = 0;  // a byte per slot: the lane whose access does
             unsigned grp[RPL];   // AGG: the lanes whose accesses this slot folds, in lane order
@@ -443,6 +457,15 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                 } else {
                     nv = step(o, q.tid[i], q.op[i], &r);
                 }
+                if (nv != o && lookup) {
+                    const unsigned key = flight_key(q.word[i], q.op[i]);
+                    const unsigned out = atomicCAS(&s_flight[flight_slot(q.word[i])], 0u, key);
+                    if (out == key) {
+                        defer |= 1u << k;
+                        continue;
+                    }
+                    own |= (unsigned)(out == 0u) << k;
+                }
                 if (nv != o) {
                     seen[k] = hr_shadow_cas(shadow, q.word[i], o, nv, g);
                     casm |= 1u << k;
@@ -468,6 +491,17 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                 } else if ((race >> (8 * k)) & 0xFFu) {
                     todo |= 1u << k;
                 }
+                if ((own >> k) & 1u) *(volatile unsigned*)&s_flight[flight_slot(q.word[i])] = 0u;
+            }
+            if (defer) {  // look again, every word's load before the first result
+#pragma unroll
+                for (int k = 0; k < RPL; ++k)
+                    if ((defer >> k) & 1u) seen[k] = hr_shadow_load(shadow, q.word[queued + k * 32 + lane], g);
+#pragma unroll
+                for (int k = 0; k < RPL; ++k)
+                    if ((defer >> k) & 1u) q.o[queued + k * 32 + lane] = seen[k];
+                lost |= defer;
+                todo |= defer;
             }
             while (todo) {
                 const unsigned k = __ffs(todo) - 1;
