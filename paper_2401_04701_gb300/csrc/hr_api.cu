@@ -256,10 +256,8 @@ static hr_status ensure_bin(RegionHost& r, uint64_t n, cudaStream_t s)
     cudaError_t e = cudaSuccess;
     if (!r.bin_mem || r.bin.seg_cap < n_seg) {
         const unsigned cap = (unsigned)((r.capacity + HR_BIN_SEG - 1) / HR_BIN_SEG);
-        unsigned clusters = 0, sub = 0;
-        hr_bin_shape(&clusters, &sub);
-        const unsigned slices = clusters * sub;
-        const unsigned part_cap = HR_BIN_MAX_WAVES + slices - 1;
+        hr_bin_shape(cap, &r.bin);
+        const unsigned part_cap = HR_BIN_MAX_WAVES + r.bin.slices - 1;
         const size_t bytes = hr_bin_table_bytes(cap, part_cap);
         if (r.bin_mem) e = cudaDeviceSynchronize();
         if (e == cudaSuccess) e = cudaFree(r.bin_mem);
@@ -279,9 +277,6 @@ static hr_status ensure_bin(RegionHost& r, uint64_t n, cudaStream_t s)
         r.bin.clear = (unsigned char*)p;
         r.bin.seg_cap = cap;
         r.bin.part_cap = part_cap;
-        r.bin.clusters = clusters;
-        r.bin.sub = sub;
-        r.bin.slices = slices;
     }
     if (r.bin.out_cap < n) {
         if (r.bin.out) e = cudaDeviceSynchronize();

@@ -423,19 +423,28 @@ __global__ void __launch_bounds__(SCAN_THREADS) hr_bin_scan(hr_work w)
 
 // ------------------------------------------------------------ 4. scatter
 //
-// Clusters of HR_BIN_CLUSTER CTAs; a cluster's slice is the slices of its CTAs
-// in the count pass, so a (cluster, wave) covers consecutive parts of the
+// Clusters of CL CTAs; a cluster's slice is consecutive slices of the count pass,
+// so a (cluster, wave) covers consecutive parts of the
 // table and owns one contiguous range per segment, starting at the table entry
 // of its first part.  The cluster walks its waves in order; for each, the
 // segment cursors are spread over the cluster's shared memory (segment s on
-// rank s % HR_BIN_CLUSTER) and every CTA appends its share of the wave's
-// records with atomics on those cursors (distributed shared memory).  One
-// bucket range per cluster is being filled at a time, so L2 holds one partly
-// written sector per (cluster, segment) and merges the 4- or 8-byte stores.
+// rank s % CL) and every CTA appends its share of the wave's records with
+// atomics on those cursors (distributed shared memory).  One bucket range per
+// cluster is being filled at a time, so L2 holds one partly written sector per
+// (cluster, segment) and merges the 4- or 8-byte stores.
+//
+// Bound by the cursors' atomics and by those open sectors.  Smaller clusters keep
+// more of the atomics in the CTA's own shared memory and fill more SMs (38 clusters
+// of 4 against 15 of 8 on 152 SMs), but open more sectors: 2^14 segments x 76
+// clusters of 2 are 40 MB, more than L2 merges beside the record stream.  Time of
+// this kernel with CL = 2, 4, 8: 2^14 segments (75.2M records) 834, 547, 607 us;
+// 2^12 (18.8M) 137, 129, 178 us; 2^10 (4.7M) 38, 49, 75 us; hence the rule of
+// hr_bin_shape().  Copying the records through shared memory two steps ahead was
+// slower (623, 140, 50 us with CL = 4): the loads are not what it waits for.
 
-constexpr unsigned CL = HR_BIN_CLUSTER;
 constexpr unsigned SCATTER_R = 4;  // records per thread per step: their atomics are in flight together
 
+template <unsigned CL>
 struct ScatterSmem {
     unsigned long long start[HR_BIN_MAX_WAVES + 1];
     unsigned long long key[HR_BIN_MAX_WAVES];
@@ -443,13 +452,13 @@ struct ScatterSmem {
     unsigned p0[HR_BIN_MAX_SUB], w0[HR_BIN_MAX_SUB], np[HR_BIN_MAX_SUB];  // the cluster's count slices
     unsigned cur[HR_BIN_MAX_SEGS / CL];
 };
-constexpr size_t SCATTER_SMEM = sizeof(ScatterSmem);
 
-__global__ void __cluster_dims__(HR_BIN_CLUSTER, 1, 1) __launch_bounds__(STREAM_THREADS)
+template <unsigned CL>
+__global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(STREAM_THREADS)
     hr_bin_scatter(hr_region_dev* __restrict__ regions, hr_work w)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    ScatterSmem& S = *reinterpret_cast<ScatterSmem*>(smem_raw);
+    auto& S = *reinterpret_cast<ScatterSmem<CL>*>(smem_raw);
     cg::cluster_group cluster = cg::this_cluster();
     if (!hr_bin_taken(w.ctl)) return;  // the same for every CTA: no remote access happens
     const unsigned W = w.ctl->n_waves, P = w.ctl->bin_parts;
@@ -939,13 +948,13 @@ cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const u
                               (const void*)hr_bin_groups<false>})
             cudaFuncSetAttribute(k, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
         cudaFuncSetAttribute(hr_bin_count, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)STREAM_SMEM);
-        cudaFuncSetAttribute(hr_bin_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
         cudaFuncSetAttribute(hr_bin_groups<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
         cudaFuncSetAttribute(hr_bin_groups<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
         g_attrs = true;
     }
     const hr_bin& b = w.bin;
     if (b.n_seg == 0 || b.n_seg > b.seg_cap || b.n_seg > HR_BIN_MAX_SEGS || b.clusters == 0 || b.sub == 0 ||
+        (b.cluster != HR_BIN_CLUSTER_FEW && b.cluster != HR_BIN_CLUSTER) ||
         b.sub > HR_BIN_MAX_SUB || b.slices != b.clusters * b.sub || b.slices > STREAM_THREADS ||
         b.part_cap < HR_BIN_MAX_WAVES + b.slices - 1)
         return cudaErrorInvalidValue;
@@ -953,7 +962,12 @@ cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const u
     hr_bin_count<<<b.slices, STREAM_THREADS, STREAM_SMEM, stream>>>(d_regions, w);
     hr_bin_scan_sums<<<scan_blocks, SCAN_THREADS, 0, stream>>>(w);
     hr_bin_scan<<<scan_blocks, SCAN_THREADS, 0, stream>>>(w);
-    hr_bin_scatter<<<b.clusters * CL, STREAM_THREADS, SCATTER_SMEM, stream>>>(d_regions, w);
+    if (b.cluster == HR_BIN_CLUSTER_FEW)
+        hr_bin_scatter<HR_BIN_CLUSTER_FEW><<<b.clusters * HR_BIN_CLUSTER_FEW, STREAM_THREADS,
+                                             sizeof(ScatterSmem<HR_BIN_CLUSTER_FEW>), stream>>>(d_regions, w);
+    else
+        hr_bin_scatter<HR_BIN_CLUSTER><<<b.clusters * HR_BIN_CLUSTER, STREAM_THREADS, sizeof(ScatterSmem<HR_BIN_CLUSTER>),
+                                         stream>>>(d_regions, w);
     static int sms = 0;  // one persistent segment CTA per SM
     if (!sms) {
         int dev = 0;
@@ -965,10 +979,12 @@ cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const u
     return cudaGetLastError();
 }
 
-// The binned checker's streaming shape: scatter clusters of HR_BIN_CLUSTER CTAs,
-// as many as can be resident at once (one CTA per SM), and count slices per
-// cluster slice so that the count pass (one CTA per SM) fills the SMs.
-void hr_bin_shape(unsigned* clusters_out, unsigned* sub_out)
+namespace {
+
+// as many clusters of CL CTAs as can be resident at once (one CTA per SM), and
+// count slices per cluster slice so that the count pass (one CTA per SM) fills the SMs
+template <unsigned CL>
+void shape_of(hr_bin* bin)
 {
     static unsigned c_cached = 0, s_cached = 0;
     if (!c_cached) {
@@ -976,11 +992,12 @@ void hr_bin_shape(unsigned* clusters_out, unsigned* sub_out)
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms < (int)CL) sms = CL;
-        cudaFuncSetAttribute(hr_bin_scatter, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SCATTER_SMEM);
+        cudaFuncSetAttribute(hr_bin_scatter<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)sizeof(ScatterSmem<CL>));
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3((unsigned)(sms / CL * CL));
         cfg.blockDim = dim3(STREAM_THREADS);
-        cfg.dynamicSmemBytes = SCATTER_SMEM;
+        cfg.dynamicSmemBytes = sizeof(ScatterSmem<CL>);
         cudaLaunchAttribute attr;
         attr.id = cudaLaunchAttributeClusterDimension;
         attr.val.clusterDim.x = CL;
@@ -989,7 +1006,7 @@ void hr_bin_shape(unsigned* clusters_out, unsigned* sub_out)
         cfg.attrs = &attr;
         cfg.numAttrs = 1;
         int clusters = 0;
-        if (cudaOccupancyMaxActiveClusters(&clusters, (void*)hr_bin_scatter, &cfg) != cudaSuccess || clusters < 1) {
+        if (cudaOccupancyMaxActiveClusters(&clusters, (void*)hr_bin_scatter<CL>, &cfg) != cudaSuccess || clusters < 1) {
             (void)cudaGetLastError();
             clusters = sms / (int)CL;
         }
@@ -997,9 +1014,21 @@ void hr_bin_shape(unsigned* clusters_out, unsigned* sub_out)
         if (sub < 1) sub = 1;
         if (sub > HR_BIN_MAX_SUB) sub = HR_BIN_MAX_SUB;
         while ((unsigned)clusters * sub > STREAM_THREADS) --sub;
-        c_cached = (unsigned)clusters;
         s_cached = sub;
+        c_cached = (unsigned)clusters;
     }
-    *clusters_out = c_cached;
-    *sub_out = s_cached;
+    bin->cluster = CL;
+    bin->clusters = c_cached;
+    bin->sub = s_cached;
+    bin->slices = c_cached * s_cached;
+}
+
+}  // namespace
+
+// The binned checker's streaming shape for a region of n_seg segments (the scatter's
+// comment has both sides measured; at 2^12 segments the two are within 6 %)
+void hr_bin_shape(unsigned n_seg, hr_bin* bin)
+{
+    if (n_seg <= HR_BIN_FEW_SEGS) shape_of<HR_BIN_CLUSTER_FEW>(bin);
+    else shape_of<HR_BIN_CLUSTER>(bin);
 }

@@ -158,7 +158,9 @@ static_assert(HR_BIN_SEG_SHIFT >= 10 && HR_BIN_SEG_SHIFT <= 13, "the packed acce
 constexpr unsigned HR_BIN_MAX_SEGS = 16384;              // larger regions take the per-wave checker
 constexpr unsigned HR_BIN_MAX_WAVES = 256;               // checks with more waves take the per-wave checker
 constexpr unsigned HR_BIN_SCAN = 4096;                   // table entries per scan block
-constexpr unsigned HR_BIN_CLUSTER = 8;                   // CTAs sharing bucket cursors in the scatter
+constexpr unsigned HR_BIN_CLUSTER = 4;                   // CTAs sharing bucket cursors in the scatter ...
+constexpr unsigned HR_BIN_CLUSTER_FEW = 2;               // ... for regions of at most HR_BIN_FEW_SEGS segments
+constexpr unsigned HR_BIN_FEW_SEGS = 2048;
 constexpr unsigned HR_BIN_MAX_SUB = 16;                  // count slices per cluster slice, at most
 struct hr_bin {
     unsigned* table;         // [seg_cap * part_cap] counts, then offsets
@@ -171,7 +173,8 @@ struct hr_bin {
     unsigned n_seg;          // segments of this check's region
     unsigned seg_cap;        // segments the table holds
     unsigned part_cap;       // parts the table holds: HR_BIN_MAX_WAVES + slices - 1
-    unsigned clusters;       // scatter clusters (hr_bin_shape())
+    unsigned cluster;        // CTAs of a scatter cluster (hr_bin_shape())
+    unsigned clusters;       // scatter clusters
     unsigned sub;            // count slices per cluster slice
     unsigned slices;         // count slices (CTAs of the count pass): clusters * sub
     unsigned pow2;           // 1: block size and warp size are powers of two (bit-operation FSM step)
@@ -320,9 +323,9 @@ constexpr unsigned HR_SMALL_INTERVALS = 4096;  // pre-pass intervals of a single
 // when they took the check.
 cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const unsigned char* d_table,
                              cudaStream_t stream);
-// The binned checker's streaming shape: as many scatter clusters as fit at once,
-// and count slices per cluster slice so that the count pass fills the SMs.
-void hr_bin_shape(unsigned* clusters, unsigned* sub);
+// The binned checker's streaming shape for a region of n_seg segments (cluster,
+// clusters, sub and slices of *bin).
+void hr_bin_shape(unsigned n_seg, hr_bin* bin);
 // bytes of a region's binned-checker tables (without the access buffer)
 inline size_t hr_bin_table_bytes(unsigned seg_cap, unsigned part_cap)
 {
