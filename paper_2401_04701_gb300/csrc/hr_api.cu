@@ -80,6 +80,9 @@ struct hr_ctx {
     unsigned cas_cap = HR_DEFAULT_CAS_CAP;
     unsigned test_flags = 0;
     unsigned variant = 0;              // kernel variant of later checks (hr_set_variant / hr_autotune)
+    bool chosen = false;               // the caller chose it; else checks may take the binned route
+    unsigned long long auto_bytes = 0; // scratch allocated for checks that took that route by themselves
+    std::vector<void*> retired;        // buffers outgrown there (checks in flight may still use them)
     cudaStream_t copies = nullptr;     // non-blocking stream for report copies (never waits on user streams)
     void* batch_mem = nullptr;         // scratch of hr_check_batch (allocated on first use)
     // hr_check_trace_host: two device staging buffers, a copy stream, and events
@@ -128,6 +131,7 @@ static void free_ctx(hr_ctx* c)
             cudaEventDestroy(p.mid);
             cudaEventDestroy(p.end);
         }
+    for (void* p : c->retired) cudaFree(p);
     if (c->copies) cudaStreamDestroy(c->copies);
     for (int b = 0; b < 2; ++b) {
         cudaFree(c->stage_buf[b]);
@@ -292,6 +296,44 @@ static hr_status ensure_bin(RegionHost& r, uint64_t n, cudaStream_t s)
     return HR_OK;
 }
 
+// Whether a check for which no variant was chosen can take the binned route: its
+// size (the pre-pass decides the rest), and scratch for it.  The scratch is
+// allocated on first use, within HR_BIN_AUTO_BYTES per context and a quarter of the
+// free memory; without it the check takes the per-wave checker.  Nothing is
+// allocated while the stream is captured, no allocation disturbs a capture in another
+// thread, and a buffer that became too small lives until the context does.
+static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
+{
+    const unsigned cap_seg = (unsigned)((r.capacity + HR_BIN_SEG - 1) / HR_BIN_SEG);
+    const uint64_t n_seg = (r.desc.n_words + HR_BIN_SEG - 1) / HR_BIN_SEG;
+    if (ctx->chosen || r.desc.report_mode == HR_REPORT_EVERY_EPOCH || n < HR_BIN_AUTO_MIN_N || n > HR_BIN_AUTO_MAX_N ||
+        n_seg < HR_BIN_AUTO_SEGS || cap_seg > HR_BIN_MAX_SEGS || ctx->test_flags || ctx->cas_cap < HR_DEFAULT_CAS_CAP)
+        return false;
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
+    if (r.bin_mem && r.bin.out_cap >= n) return ensure_bin(r, n, s) == HR_OK;
+    hr_bin shape{};
+    hr_bin_shape(cap_seg, &shape);
+    const uint64_t room = (n + n / 8 + 0xFFFFF) & ~0xFFFFFull;  // calls of about one size share a buffer
+    const uint64_t bytes = room * sizeof(uint2) + (r.bin_mem ? 0 : hr_bin_table_bytes(cap_seg, HR_BIN_MAX_WAVES + shape.slices - 1));
+    size_t free_b = 0, total_b = 0;
+    if (ctx->auto_bytes + bytes > HR_BIN_AUTO_BYTES || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
+        bytes > free_b / 4) {
+        (void)cudaGetLastError();
+        return false;
+    }
+    cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+    if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
+    if (r.bin.out) ctx->retired.push_back(r.bin.out);
+    r.bin.out = nullptr;
+    r.bin.out_cap = 0;
+    const bool ok = ensure_bin(r, room, s) == HR_OK;
+    cudaThreadExchangeStreamCaptureMode(&mode);
+    if (ok) ctx->auto_bytes += bytes;
+    else (void)cudaGetLastError();
+    return ok;
+}
+
 static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_trace, uint64_t n,
                               uint32_t kernel_base, hr_stream_t stream, bool aggregate)
 {
@@ -327,6 +369,9 @@ static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_t
         const hr_status bs = ensure_bin(r, n, s);
         if (bs != HR_OK) return bs;
         w.bin = r.bin;
+    } else if (aggregate && auto_binned(ctx, r, n, s)) {
+        w.bin = r.bin;
+        w.bin.automatic = 1u;
     }
     unsigned launches = 0;
     cudaError_t e = hr_launch_jobs(ctx->d_regions, w, &job, 1, ctx->d_table, variant, s,
@@ -665,6 +710,7 @@ extern "C" hr_status hr_set_variant(hr_ctx* ctx, uint32_t id)
 {
     if (!ctx || id >= HR_N_VARIANTS) return HR_ERR_INVALID;
     ctx->variant = id;
+    ctx->chosen = true;
     return HR_OK;
 }
 
@@ -686,6 +732,8 @@ extern "C" hr_status hr_autotune(hr_ctx* ctx, uint32_t region, const hr_record* 
     cudaError_t e = cudaEventCreate(&a);
     if (e == cudaSuccess) e = cudaEventCreate(&b);
     const unsigned saved = ctx->variant;
+    const bool saved_chosen = ctx->chosen;
+    ctx->chosen = true;
     const bool saved_profile = ctx->profile;
     ctx->profile = false;
     float best_ms = 0.0f;
@@ -725,6 +773,7 @@ extern "C" hr_status hr_autotune(hr_ctx* ctx, uint32_t region, const hr_record* 
     }
     ctx->profile = saved_profile;
     ctx->variant = (st == HR_OK && e == cudaSuccess) ? best_v : saved;
+    if (st != HR_OK || e != cudaSuccess) ctx->chosen = saved_chosen;
     if (best) *best = ctx->variant;
     if (a) cudaEventDestroy(a);
     if (b) cudaEventDestroy(b);

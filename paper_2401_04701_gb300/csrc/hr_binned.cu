@@ -68,7 +68,7 @@ constexpr unsigned PACK4_TID_LIMIT = 1u << (32 - PACK4_TID_SHIFT);
 // results; every kernel below decides the same way)
 __device__ __forceinline__ bool bin_fits(const hr_ctl* c)
 {
-    return c->n_jobs == 1 && c->total_items > 0 && c->n_waves >= 1 && c->n_waves <= HR_BIN_MAX_WAVES;
+    return !c->bin_skip && c->n_jobs == 1 && c->total_items > 0 && c->n_waves >= 1 && c->n_waves <= HR_BIN_MAX_WAVES;
 }
 
 __device__ __forceinline__ uint32_t smem_addr(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
@@ -315,7 +315,10 @@ __global__ void __launch_bounds__(STREAM_THREADS) hr_bin_count(hr_region_dev* __
         for (unsigned i = tx; i < n_seg; i += STREAM_THREADS) w.bin.table[(size_t)i * P + part] = S.seg[i];
         __syncthreads();
     }
-    if (err) hr_set_error(&rg->error, err);
+    if (err) {
+        if (w.bin.automatic) w.ctl->bin_err = 1u;
+        else hr_set_error(&rg->error, err);
+    }
     // the largest thread id decides the packing of the bucketed accesses
     for (int o = 16; o > 0; o >>= 1) max_tid = max(max_tid, __shfl_xor_sync(0xFFFFFFFFu, max_tid, o));
     if (lane == 0 && max_tid) atomicMax(&w.ctl->bin_max_tid, max_tid);

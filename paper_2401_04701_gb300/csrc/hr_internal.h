@@ -130,6 +130,9 @@ struct hr_ctl {
     unsigned seg_ticket;   // binned checker: next segment a thread group of the segment pass takes
     unsigned bin_max_seg;  // binned checker: accesses of the fullest segment
     unsigned bin_count;    // binned checker: accesses counted into buckets
+    unsigned bin_skip;     // automatic route: 1: the pre-pass left this check to the per-wave checker
+    unsigned bin_err;      // automatic route: 1: the count pass met an error (the per-wave checker then
+                           // does the check, and reports it)
 };
 
 // Whether the binned checker applies this check (the flag, and the skew guard:
@@ -139,8 +142,32 @@ struct hr_ctl {
 // binned kernels).  Read by the kernels after the count and scan passes.
 __host__ __device__ inline bool hr_bin_taken(const hr_ctl* c)
 {
-    return c->binned && !(c->bin_count >= HR_BIN_SKEW_MIN && (unsigned long long)c->bin_max_seg * HR_BIN_SKEW > c->bin_count);
+    return c->binned && !c->bin_err && !(c->bin_count >= HR_BIN_SKEW_MIN && (unsigned long long)c->bin_max_seg * HR_BIN_SKEW > c->bin_count);
 }
+
+// The automatic route: a check for which no variant was chosen takes the binned
+// checker when its pre-pass expects that to be faster, and the count pass meets no
+// error.  The expectation, in picoseconds: the per-wave checker
+// needs about 9 us a wave and 28 ps a record; the binned one 75 us, 18 ps a record,
+// 2.4 ps a word of the region (its shadow is written, and read unless nothing in it
+// is live) and 1.6 ns an access of the fullest segment (one thread group applies
+// it), which a sample of the records estimates.  Measured on global-memory traces
+// (us a call, pre-pass included, per-wave variant 0 / binned): 32 waves, 0.29M
+// records on 2^20 words 289 / 100, 1.18M 296 / 112, 4.7M on 2^22 words 362 / 151,
+// 75.2M on 2^26 words 2145 / 1304; 8 waves, 1.18M on 2^22 words 113 / 103; 4 waves,
+// 0.59M on 2^22 words 70 / 87, 2.35M on 2^24 words 109 / 152; 1 wave, 2.35M on
+// 2^26 words 95 / 267.  A check that the pre-pass leaves to the per-wave checker
+// pays about 20 us for the binned kernels that find nothing to do; that counts on the
+// per-wave checker's side, and smaller checks and regions never get there.
+constexpr unsigned long long HR_BIN_AUTO_MIN_N = 1ull << 18;     // records
+constexpr unsigned long long HR_BIN_AUTO_MAX_N = 1ull << 27;     // (1 GiB of bucketed accesses)
+constexpr unsigned long long HR_BIN_AUTO_BYTES = 3ull << 30;     // scratch a context allocates for it, at most
+constexpr unsigned HR_BIN_AUTO_SEGS = 256;
+constexpr unsigned HR_BIN_SAMPLES = 4096;                        // records sampled
+constexpr unsigned long long HR_BIN_AUTO_PS_WAVE = 9000000, HR_BIN_AUTO_PS_REC = 28, HR_BIN_AUTO_PS_SKIP = 20000000,
+                             HR_BIN_AUTO_PS_BIN = 75000000,
+                             HR_BIN_AUTO_PS_BIN_REC = 18, HR_BIN_AUTO_PS_BIN_5_WORDS = 12,
+                             HR_BIN_AUTO_PS_BIN_FULLEST = 1600;
 
 // Scratch of the binned checker (hr_binned.cu), one per region.  The region's
 // shadow is cut into segments of HR_BIN_SEG words.  The trace is cut into one
@@ -177,6 +204,7 @@ struct hr_bin {
     unsigned clusters;       // scatter clusters
     unsigned sub;            // count slices per cluster slice
     unsigned slices;         // count slices (CTAs of the count pass): clusters * sub
+    unsigned automatic;      // 1: no variant was chosen; the check takes this route where it is faster
     unsigned pow2;           // 1: block size and warp size are powers of two (bit-operation FSM step)
 };
 
@@ -201,7 +229,7 @@ struct hr_work {
     unsigned test_flags;             // HR_TEST_* hooks (tests only)
     unsigned views;                  // 1: a device view of the checked region exists (inline writes may
                                      // carry kernel ordinals the region's last key does not know)
-    hr_bin bin;                      // binned checker scratch (variant HR_BIN_VARIANT only)
+    hr_bin bin;                      // binned checker scratch (variant HR_BIN_VARIANT and the automatic route)
 };
 
 constexpr unsigned long long HR_DEFAULT_WAIT_NS = 4000000000ull;  // 4 s

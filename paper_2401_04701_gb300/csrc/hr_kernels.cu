@@ -174,6 +174,8 @@ __device__ void scan_counts_body(hr_work& w, unsigned total_int, hr_region_dev* 
         w.ctl->bin_max_tid = 0;
         w.ctl->bin_max_seg = 0;
         w.ctl->bin_count = 0;
+        w.ctl->bin_skip = 0;
+        w.ctl->bin_err = 0;
         w.ctl->n_waves = over ? 0u : (unsigned)total;
     }
 }
@@ -415,12 +417,57 @@ __device__ __forceinline__ bool interval_boundaries(const hr_record* t, unsigned
     return ordered;
 }
 
+// Whether the automatic route leaves this check to the per-wave checker (the rule
+// beside HR_BIN_AUTO_MIN_N).  The fullest segment's accesses are estimated from one
+// record at a scattered place of each of HR_BIN_SAMPLES equal parts of the trace,
+// counted per segment (per run of segments when there are more than counters).
+// hist: HR_BIN_SAMPLES counters in shared memory.
+__device__ void bin_choose(hr_work& w, const hr_jobd& jb, const hr_region_dev& rg, unsigned* hist)
+{
+    const unsigned waves = w.ctl->n_waves;
+    const unsigned long long per_wave =
+        HR_BIN_AUTO_PS_SKIP + waves * HR_BIN_AUTO_PS_WAVE + jb.n * HR_BIN_AUTO_PS_REC;
+    const unsigned long long binned =
+        HR_BIN_AUTO_PS_BIN + jb.n * HR_BIN_AUTO_PS_BIN_REC + rg.n_words / 5 * HR_BIN_AUTO_PS_BIN_5_WORDS;
+    if (waves > HR_BIN_MAX_WAVES || binned >= per_wave) {  // the same for every thread
+        if (threadIdx.x == 0) w.ctl->bin_skip = 1u;
+        return;
+    }
+    __shared__ unsigned s_fullest;
+    if (threadIdx.x == 0) s_fullest = 0u;
+    for (unsigned i = threadIdx.x; i < HR_BIN_SAMPLES; i += blockDim.x) hist[i] = 0u;
+    __syncthreads();
+    const bool filtering = hr_filter_active(rg.filter);
+    const unsigned n_seg = w.bin.n_seg;
+    const unsigned long long part = jb.n / HR_BIN_SAMPLES;  // >= 1: n >= HR_BIN_AUTO_MIN_N
+    unsigned fullest = 0;
+#pragma unroll 4
+    for (unsigned i = threadIdx.x; i < HR_BIN_SAMPLES; i += blockDim.x) {
+        const unsigned long long at = i * part + (i * 2654435761u) % (unsigned)part;
+        const uint4 v = __ldg(reinterpret_cast<const uint4*>(jb.trace + at));
+        unsigned tid = v.y;
+        unsigned long long idx = v.x;
+        if (((v.w >> 16) & 0xFFu) > HR_A || (filtering && !hr_monitored(rg.filter, rg.geom, &tid, v.x, &idx)) ||
+            idx >= rg.n_words)
+            continue;
+        const unsigned seg = (unsigned)(idx >> HR_BIN_SEG_SHIFT);
+        const unsigned b = n_seg > HR_BIN_SAMPLES ? (unsigned)((unsigned long long)seg * HR_BIN_SAMPLES / n_seg) : seg;
+        fullest = max(fullest, atomicAdd(&hist[b], 1u) + 1u);
+    }
+    if (fullest) atomicMax(&s_fullest, fullest);
+    __syncthreads();
+    if (threadIdx.x == 0 && binned + s_fullest * part * HR_BIN_AUTO_PS_BIN_FULLEST >= per_wave) w.ctl->bin_skip = 1u;
+}
+static_assert(HR_BIN_AUTO_MAX_N / HR_BIN_SAMPLES < (1ull << 32) && HR_BIN_AUTO_MIN_N >= HR_BIN_SAMPLES, "sample parts");
+static_assert(HR_BIN_SAMPLES <= HR_SMALL_INTERVALS, "the sample's counters fit the interval list");
+
 // The whole pre-pass of one small trace (at most HR_SMALL_INTERVALS intervals)
 // in one CTA: the four kernels above as phases separated by block barriers, so
 // a small check costs two launches instead of five.  Phase (a) finds the
 // intervals holding a wave boundary (one lane per interval, two keys each),
 // (b) counts each one's boundaries (a warp per interval), (c) scans the counts,
-// (d) writes the wave table, (e) builds the stages.
+// (d) writes the wave table, (e) builds the stages, (f) chooses the checker when
+// the caller left that open.
 __global__ void __launch_bounds__(1024) hr_prepass_small(const JobParams<1> P, unsigned total_int, hr_work w,
                                                          hr_region_dev* regions)
 {
@@ -480,6 +527,11 @@ __global__ void __launch_bounds__(1024) hr_prepass_small(const JobParams<1> P, u
     __syncthreads();
     // (e)
     stages_one_job(w, regions);
+    // (f)
+    if (w.bin.automatic) {
+        __syncthreads();
+        bin_choose(w, jb, regions[jb.region], s_list);
+    }
 }
 
 // ------------------------------------------------------------ the FSM checker
@@ -1218,9 +1270,10 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
                            cudaEvent_t before_check, unsigned* launches)
 {
     if (variant > HR_EVERY_EPOCH_VARIANT) return cudaErrorInvalidValue;
-    const bool binned = variant == HR_BIN_VARIANT;
+    const bool binned = variant == HR_BIN_VARIANT || w_in.bin.automatic;
     if (binned && (n_jobs != 1 || !w_in.bin.table)) return cudaErrorInvalidValue;
-    if (binned) variant = HR_BIN_FALLBACK;  // the per-wave checker runs after it (and finds no work when binned)
+    // the per-wave checker runs after it (and finds no work when binned)
+    if (variant == HR_BIN_VARIANT) variant = HR_BIN_FALLBACK;
     hr_work w = w_in;
     const bool runs = n_jobs == 1 && hr_variant_runs(variant);
     w.tile = runs ? hr_run_tile(variant) : hr_variant_tile(variant);
@@ -1238,6 +1291,7 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
             hr_prepass_small<<<1, 1024, 0, stream>>>(P, total_int, w, d_regions);
             prepass_launches = 1;
         } else {
+            if (w.bin.automatic) return cudaErrorInvalidValue;  // the choice is made in the one-CTA pre-pass
             launch_prepass(P, total_int, d_regions, w, stream);
         }
     } else {
