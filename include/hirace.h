@@ -179,7 +179,7 @@ hr_status hr_check_trace(hr_ctx* ctx, uint32_t region, const hr_record* d_trace,
 
 /*
  * hr_check_trace_host - hr_check_trace over a trace in HOST memory: the trace
- * is copied in chunks of chunk_records records (0: 2^24, i.e. 256 MB) through
+ * is copied in chunks of chunk_records records (0: 2^21, i.e. 32 MB) through
  * two device staging buffers owned by the context, each chunk's copy (on a
  * copy stream of the context) overlapping the check of the chunk before it on
  * `stream`.  Chunks may cut waves (the shadow stays resident between them).

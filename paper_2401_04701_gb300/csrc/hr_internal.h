@@ -56,6 +56,7 @@ struct hr_region_dev {
     unsigned long long n_races;   // races found (may exceed ring_cap)
     unsigned int error;           // sticky first error (hr_status)
     unsigned int flags;           // HR_FLAG_* bits
+    unsigned long long group_waves;  // waves of the record group a host-memory check is in (hr_work::cont)
     unsigned long long last_key;  // wave key after the region's last processed record
     unsigned int used;            // 1: a record was processed since init/reset; 2: the shadow's
                                   // contents are unknown (cleared before the first wave)
@@ -229,6 +230,8 @@ struct hr_work {
     unsigned test_flags;             // HR_TEST_* hooks (tests only)
     unsigned views;                  // 1: a device view of the checked region exists (inline writes may
                                      // carry kernel ordinals the region's last key does not know)
+    unsigned cont;                   // 1: goes on with the record group of the region's last check, whose
+                                     // waves count together against max_waves (single-trace checks only)
     hr_bin bin;                      // binned checker scratch (variant HR_BIN_VARIANT and the automatic route)
 };
 

@@ -155,7 +155,13 @@ __device__ void scan_counts_body(hr_work& w, unsigned total_int, hr_region_dev* 
     }
     __syncthreads();
     const unsigned n_jobs = w.ctl->n_jobs;
-    const bool over = total > w.max_waves;
+    unsigned long long waves = total;
+    if (w.cont) {
+        const hr_jobd& jb = w.jobs[0];
+        const hr_region_dev& rg = regions[jb.region];
+        waves += rg.group_waves - (key_at(jb.trace, 0, jb.kb) == rg.last_key);  // (a wave cut in two counts once)
+    }
+    const bool over = waves > w.max_waves;
     for (unsigned j = threadIdx.x; j < n_jobs; j += blockDim.x) {
         hr_jobd& jb = w.jobs[j];
         const unsigned first = w.counts[jb.int_begin];
@@ -294,6 +300,7 @@ __device__ void stages_one_job(hr_work& w, hr_region_dev* regions)
         w.ctl->fresh = !failed && nw > 0 && !w.views &&
                        (rg.used != 1 || (w.wave_key[jb.wave_begin] >> 32) > (rg.last_key >> 32));
         if (!failed && nw > 0) {
+            rg.group_waves = nw + (w.cont ? rg.group_waves - (w.wave_key[jb.wave_begin] == rg.last_key) : 0ull);
             rg.last_key = w.wave_key[jb.wave_begin + nw - 1];
             rg.used = 1;
         }

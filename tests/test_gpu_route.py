@@ -112,3 +112,15 @@ def test_errors_as_the_per_wave_checker_has_them(hr, what):
     assert hr.STATUS[got[0]] == hr.STATUS[want[0]] == "HR_ERR_" + what.upper()
     clean = check(hr, trace_of(6), reg, {}, 1, 3)
     assert 0.9 * clean[1] < got[1] <= clean[1]
+
+
+def test_host_trace_wave_limit_counts_over_pieces(hr, monkeypatch):
+    """By default a host trace travels in pieces of 2^21 records; the limit of waves per call still
+    holds for each 2^24 records together."""
+    import torch
+    monkeypatch.setenv("HR_MAX_WAVES", "8")
+    for waves, status in ((8, "HR_OK"), (9, "HR_ERR_CAPACITY")):
+        trace = trace_of(waves, n=(1 << 22) + 99, waves=waves)   # three pieces, at most 5 waves each
+        with hr.Checker([dict(n_words=WORDS, block_dim=64)]) as ck:
+            ck.check_trace_host(0, torch.from_numpy(trace.view(np.uint8)).pin_memory())
+            assert hr.STATUS[ck.report(0, cap=0)[1]] == status
