@@ -530,7 +530,8 @@ extern "C" hr_status hr_check_batch(hr_ctx* ctx, const hr_job* jobs, uint32_t n_
         if (st != HR_OK) return st;
     }
     // split the pre-pass interval budget across the jobs
-    const unsigned budget = HR_BATCH_INTERVALS / (unsigned)js.size();
+    const unsigned share = HR_BATCH_INTERVALS / (unsigned)js.size();
+    const unsigned budget = share < HR_SMALL_INTERVALS ? share : HR_SMALL_INTERVALS;
     unsigned at = 0;
     for (auto& d : js) {
         hr_plan_intervals(d.n, budget, &d.G, &d.n_int);

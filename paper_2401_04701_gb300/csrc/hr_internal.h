@@ -213,7 +213,7 @@ struct hr_bin {
 // table, stage list and control block.
 struct hr_work {
     hr_jobd* jobs;                   // [max_jobs]
-    unsigned* counts;                // [max_intervals] boundaries per interval, then their offsets
+    unsigned* counts;                // [max_intervals] boundaries per interval, then offsets among the job's waves
     unsigned long long* wave_start;  // [max_waves] first record (index into the job's trace)
     unsigned long long* wave_end;    // [max_waves] one past the last record
     unsigned long long* wave_key;    // [max_waves] rebased wave key
@@ -337,8 +337,8 @@ constexpr unsigned long long HR_KEY_MASK = 0xFFFFFFFFFFFFull;
 // kernel launch helpers (hr_kernels.cu)
 // Check n_jobs jobs (1..HR_MAX_BATCH) on the regions of d_regions with the
 // scratch w.  Jobs must name distinct regions and hold n > 0 records.
-// *launches (if not NULL) receives the kernels launched: 2 for a small single
-// trace (one-CTA pre-pass), 5 otherwise.
+// *launches (if not NULL) receives the kernels launched: 2 for a single trace
+// (7 with the binned checker), 4 for a batch.
 cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w, const hr_jobd* jobs, unsigned n_jobs,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream,
                            cudaEvent_t before_check, unsigned* launches = nullptr);
@@ -348,7 +348,8 @@ cudaError_t hr_launch_runs(hr_region_dev* d_regions, const hr_work& w, unsigned 
 // interval size and count for a job of n records when it may use up to budget intervals
 void hr_plan_intervals(unsigned long long n, unsigned budget, unsigned* G, unsigned* n_int);
 int hr_check_grid_size(unsigned variant);
-constexpr unsigned HR_SMALL_INTERVALS = 4096;  // pre-pass intervals of a single trace (the one-CTA pre-pass)
+constexpr unsigned HR_SMALL_INTERVALS = 4096;  // pre-pass intervals of a trace, at most (one CTA finds its waves)
+constexpr unsigned long long HR_RESET_FUSED = 4ull << 20;  // shadow bytes that a reset's one kernel clears itself
 // The binned checker's five launches (hr_binned.cu), queued after the pre-pass
 // of a single-job check; the per-wave checker queued after them finds no items
 // when they took the check.

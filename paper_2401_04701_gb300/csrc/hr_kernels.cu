@@ -1,18 +1,16 @@
 // hr_kernels.cu - the trace checker's device code (sm_103a).
 //
 // A check covers one or more jobs (a job = one trace on one region).  It runs
-// five launches on the caller's stream:
-//   1. hr_scan_intervals : per pre-pass interval of a job's trace, count the
-//                          wave boundaries (a wave is a run of equal
-//                          (kernel, bc, wc) keys); an interval is read only
-//                          when its two end keys differ
-//   2. hr_scan_counts    : exclusive scan of the counts (one CTA): global wave
-//                          numbers, each job's first wave and wave count
-//   3. hr_write_waves    : wave start offsets and keys
-//   4. hr_build_stages   : work stages per wave, an optional shadow clear
-//                          (kernel-tag group change) then the record tiles;
-//                          several jobs are interleaved wave-major
-//   5. hr_check_kernel   : persistent CTAs take work items in ticket order; a
+// on the caller's stream
+//   - the pre-pass: the waves of every trace (a wave is a run of equal (kernel,
+//     bc, wc) keys) and the work stages of every wave, an optional shadow clear
+//     (kernel-tag group change) then the record tiles.  A trace's interval is
+//     looked into only when its two end keys differ.  One trace: one CTA
+//     (hr_prepass_single).  A batch: a CTA per job counts its waves
+//     (hr_batch_count), another writes them once all counts are known
+//     (hr_batch_waves), and one CTA interleaves the jobs' stages wave-major
+//     (hr_build_stages).
+//   - hr_check_kernel   : persistent CTAs take work items in ticket order; a
 //                          stage waits (bounded) for the previous stage of the
 //                          same job, so every region sees its waves in wave
 //                          order: an order consistent with happens-before
@@ -42,72 +40,7 @@ __device__ __forceinline__ unsigned long long key_at(const hr_record* t, unsigne
     return (__ldg(p) & HR_KEY_MASK) + kb;
 }
 
-// job holding global pre-pass interval i (jobs sorted by int_begin)
-template <unsigned CAP>
-__device__ __forceinline__ unsigned job_of_interval(const JobParams<CAP>& P, unsigned i)
-{
-    unsigned lo = 0, hi = P.n;
-    while (hi - lo > 1) {
-        const unsigned mid = (lo + hi) >> 1;
-        if (P.job[mid].int_begin <= i) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 // ------------------------------------------------------------ wave discovery
-
-template <unsigned CAP>
-__global__ void hr_scan_intervals(const JobParams<CAP> P, unsigned total_int, hr_work w,
-                                  hr_region_dev* __restrict__ regions)
-{
-    const unsigned lane = threadIdx.x & 31;
-    const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const unsigned n_warps = (gridDim.x * blockDim.x) >> 5;
-    if (blockIdx.x == 0) {
-        for (unsigned j = threadIdx.x; j < P.n; j += blockDim.x) {
-            hr_jobd jb = P.job[j];
-            jb.done_ns = 0;
-            w.jobs[j] = jb;
-        }
-        if (threadIdx.x == 0) {
-            w.ctl->n_jobs = P.n;
-            w.ctl->t0_ns = globaltimer();
-        }
-    }
-    for (unsigned i = warp; i < total_int; i += n_warps) {
-        const unsigned j = job_of_interval(P, i);
-        const hr_jobd& jb = P.job[j];
-        const hr_record* trace = jb.trace;
-        const unsigned long long n = jb.n, kb = jb.kb;
-        const unsigned local = i - jb.int_begin;
-        const unsigned long long beg = (unsigned long long)local * jb.G;
-        const unsigned long long end = min(n, beg + jb.G);
-        int need = 0;
-        if (lane == 0) need = (local == 0) || key_at(trace, beg - 1, kb) != key_at(trace, end - 1, kb);
-        need = __shfl_sync(0xffffffffu, need, 0);
-        unsigned cnt = 0;
-        if (need) {
-            bool bad = false;
-#pragma unroll 8
-            for (unsigned long long c = beg; c < end; c += 32) {
-                const unsigned long long p = c + lane;
-                if (p < end) {
-                    const unsigned long long k = key_at(trace, p, kb);
-                    if (p == 0) {
-                        cnt++;
-                    } else {
-                        const unsigned long long kp = key_at(trace, p - 1, kb);
-                        cnt += k != kp;
-                        bad |= k < kp;
-                    }
-                }
-            }
-            if (bad) hr_set_error(&regions[jb.region].error, HR_ERR_ORDER);
-            for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
-        }
-        if (lane == 0) w.counts[i] = cnt;
-    }
-}
 
 // block-wide exclusive scan of one value per thread (blockDim.x == 1024)
 __device__ unsigned long long block_exclusive_scan(unsigned long long v, unsigned long long* total)
@@ -136,99 +69,40 @@ __device__ unsigned long long block_exclusive_scan(unsigned long long v, unsigne
     return before;
 }
 
-// Exclusive scan of the interval counts into wave offsets, each job's wave range,
-// the control block's reset (one CTA of 1024 threads).
-__device__ void scan_counts_body(hr_work& w, unsigned total_int, hr_region_dev* regions)
+// Exclusive scan of a job's interval counts into offsets among its waves; returns
+// the number of its waves (one CTA of 1024 threads).
+__device__ unsigned scan_counts(unsigned* counts, unsigned n_int)
 {
-    const unsigned per = (total_int + 1023) / 1024;
-    const unsigned b = threadIdx.x * per, e = min(total_int, b + per);
+    const unsigned per = (n_int + 1023) / 1024;
+    const unsigned b = threadIdx.x * per, e = min(n_int, b + per);
     unsigned local = 0;
-#pragma unroll 8
-    for (unsigned i = b; i < e; ++i) local += w.counts[i];
+    for (unsigned i = b; i < e; ++i) local += counts[i];
     unsigned long long total;
     unsigned run = (unsigned)block_exclusive_scan(local, &total);
-#pragma unroll 8
     for (unsigned i = b; i < e; ++i) {
-        const unsigned c = w.counts[i];
-        w.counts[i] = run;
+        const unsigned c = counts[i];
+        counts[i] = run;
         run += c;
     }
     __syncthreads();
-    const unsigned n_jobs = w.ctl->n_jobs;
-    unsigned long long waves = total;
-    if (w.cont) {
-        const hr_jobd& jb = w.jobs[0];
-        const hr_region_dev& rg = regions[jb.region];
-        waves += rg.group_waves - (key_at(jb.trace, 0, jb.kb) == rg.last_key);  // (a wave cut in two counts once)
-    }
-    const bool over = waves > w.max_waves;
-    for (unsigned j = threadIdx.x; j < n_jobs; j += blockDim.x) {
-        hr_jobd& jb = w.jobs[j];
-        const unsigned first = w.counts[jb.int_begin];
-        const unsigned next = jb.int_begin + jb.n_int < total_int ? w.counts[jb.int_begin + jb.n_int] : (unsigned)total;
-        jb.wave_begin = over ? 0u : first;
-        jb.n_waves = over ? 0u : next - first;
-        if (over) hr_set_error(&regions[jb.region].error, HR_ERR_CAPACITY);
-    }
-    if (threadIdx.x == 0) {
-        w.ctl->ticket = 0;
-        w.ctl->abort = 0;
-        w.ctl->total_items = 0;
-        w.ctl->n_stages = 0;
-        w.ctl->binned = 0;
-        w.ctl->fresh = 0;
-        w.ctl->bin_max_tid = 0;
-        w.ctl->bin_max_seg = 0;
-        w.ctl->bin_count = 0;
-        w.ctl->bin_skip = 0;
-        w.ctl->bin_err = 0;
-        w.ctl->n_waves = over ? 0u : (unsigned)total;
-    }
+    return (unsigned)total;
 }
 
-__global__ void __launch_bounds__(1024) hr_scan_counts(hr_work w, unsigned total_int, hr_region_dev* regions)
+// the control block at the start of a check
+__device__ void reset_ctl(hr_ctl* c, unsigned n_waves)
 {
-    scan_counts_body(w, total_int, regions);
-}
-
-template <unsigned CAP>
-__global__ void hr_write_waves(const JobParams<CAP> P, unsigned total_int, hr_work w)
-{
-    const unsigned lane = threadIdx.x & 31;
-    const unsigned warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const unsigned n_warps = (gridDim.x * blockDim.x) >> 5;
-    const unsigned n_waves = w.ctl->n_waves;
-    if (n_waves == 0) return;
-    for (unsigned i = warp; i < total_int; i += n_warps) {
-        const unsigned j = job_of_interval(P, i);
-        const hr_jobd& jb = P.job[j];
-        const unsigned long long kb = jb.kb;
-        const unsigned local = i - jb.int_begin;
-        const unsigned long long beg = (unsigned long long)local * jb.G;
-        const unsigned long long end = min(jb.n, beg + jb.G);
-        const unsigned next = (i + 1 < total_int) ? w.counts[i + 1] : n_waves;
-        unsigned off = w.counts[i];
-        if (off == next) continue;  // no boundary in this interval
-#pragma unroll 8
-        for (unsigned long long c = beg; c < end; c += 32) {
-            const unsigned long long p = c + lane;
-            bool is_b = false;
-            unsigned long long k = 0;
-            if (p < end) {
-                k = key_at(jb.trace, p, kb);
-                is_b = (p == 0) || k != key_at(jb.trace, p - 1, kb);
-            }
-            const unsigned mask = __ballot_sync(0xffffffffu, is_b);
-            if (is_b) {
-                const unsigned slot = off + __popc(mask & ((1u << lane) - 1u));
-                if (slot < n_waves) {
-                    w.wave_start[slot] = p;
-                    w.wave_key[slot] = k;
-                }
-            }
-            off += __popc(mask);
-        }
-    }
+    c->ticket = 0;
+    c->abort = 0;
+    c->total_items = 0;
+    c->n_stages = 0;
+    c->binned = 0;
+    c->fresh = 0;
+    c->bin_max_tid = 0;
+    c->bin_max_seg = 0;
+    c->bin_count = 0;
+    c->bin_skip = 0;
+    c->bin_err = 0;
+    c->n_waves = n_waves;
 }
 
 // stage and item counts of wave L of a job, and whether it starts with a clear
@@ -314,6 +188,20 @@ __device__ void stages_many_jobs(hr_work& w, hr_region_dev* regions)
 {
     const unsigned n_jobs = w.ctl->n_jobs;
     const unsigned j = threadIdx.x;
+    {
+        unsigned long long total;
+        const unsigned long long before = block_exclusive_scan(j < n_jobs ? w.jobs[j].n_waves : 0u, &total);
+        const bool over = total > w.max_waves;
+        if (j < n_jobs) {
+            w.jobs[j].wave_begin = over ? 0u : (unsigned)before;
+            if (over) {
+                w.jobs[j].n_waves = 0;
+                hr_set_error(&regions[w.jobs[j].region].error, HR_ERR_CAPACITY);
+            }
+        }
+        if (j == 0) reset_ctl(w.ctl, over ? 0u : (unsigned)total);
+        __syncthreads();
+    }
     hr_jobd jb{};
     bool failed = true;
     unsigned nw = 0;
@@ -371,10 +259,7 @@ __device__ void stages_many_jobs(hr_work& w, hr_region_dev* regions)
 
 __global__ void __launch_bounds__(1024) hr_build_stages(hr_work w, hr_region_dev* regions)
 {
-    if (w.ctl->n_jobs == 1)
-        stages_one_job(w, regions);
-    else
-        stages_many_jobs(w, regions);
+    stages_many_jobs(w, regions);
 }
 
 // The wave boundaries of records [beg, end) of a trace (a boundary is a
@@ -468,76 +353,122 @@ __device__ void bin_choose(hr_work& w, const hr_jobd& jb, const hr_region_dev& r
 static_assert(HR_BIN_AUTO_MAX_N / HR_BIN_SAMPLES < (1ull << 32) && HR_BIN_AUTO_MIN_N >= HR_BIN_SAMPLES, "sample parts");
 static_assert(HR_BIN_SAMPLES <= HR_SMALL_INTERVALS, "the sample's counters fit the interval list");
 
-// The whole pre-pass of one small trace (at most HR_SMALL_INTERVALS intervals)
-// in one CTA: the four kernels above as phases separated by block barriers, so
-// a small check costs two launches instead of five.  Phase (a) finds the
-// intervals holding a wave boundary (one lane per interval, two keys each),
-// (b) counts each one's boundaries (a warp per interval), (c) scans the counts,
-// (d) writes the wave table, (e) builds the stages, (f) chooses the checker when
-// the caller left that open.
-__global__ void __launch_bounds__(1024) hr_prepass_small(const JobParams<1> P, unsigned total_int, hr_work w,
-                                                         hr_region_dev* regions)
+// The waves of one trace of at most HR_SMALL_INTERVALS intervals, counted by one
+// CTA: (a) the intervals holding a wave boundary (one lane per interval, two keys
+// each) go to the list, (b) a warp per listed interval counts its boundaries,
+// (c) the counts become offsets.  counts: the job's; returns its waves.
+struct IntervalList {
+    unsigned at[HR_SMALL_INTERVALS], n;
+};
+__device__ unsigned count_waves(const hr_jobd& jb, unsigned* counts, IntervalList& list, hr_region_dev* regions)
 {
-    __shared__ unsigned s_list[HR_SMALL_INTERVALS];  // intervals holding a boundary
-    __shared__ unsigned s_n;
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const hr_jobd& jb = P.job[0];
     const unsigned long long n = jb.n, kb = jb.kb, G = jb.G;
-    if (threadIdx.x == 0) {
-        hr_jobd j0 = jb;
-        j0.done_ns = 0;
-        w.jobs[0] = j0;
-        w.ctl->n_jobs = 1;
-        w.ctl->t0_ns = globaltimer();
-        s_n = 0;
-    }
+    if (threadIdx.x == 0) list.n = 0;
     __syncthreads();
-    // (a)
-    for (unsigned i = threadIdx.x; i < total_int; i += blockDim.x) {
+    for (unsigned i = threadIdx.x; i < jb.n_int; i += blockDim.x) {
         const unsigned long long beg = (unsigned long long)i * G, end = min(n, beg + G);
         if (i == 0 || key_at(jb.trace, beg - 1, kb) != key_at(jb.trace, end - 1, kb))
-            s_list[atomicAdd(&s_n, 1u)] = i;
+            list.at[atomicAdd(&list.n, 1u)] = i;
         else
-            w.counts[i] = 0;
+            counts[i] = 0;
     }
     __syncthreads();
-    const unsigned n_need = s_n;
-    // (b)
-    for (unsigned q = warp; q < n_need; q += blockDim.x >> 5) {
-        const unsigned i = s_list[q];
+    for (unsigned q = warp; q < list.n; q += blockDim.x >> 5) {
+        const unsigned i = list.at[q];
         const unsigned long long beg = (unsigned long long)i * G, end = min(n, beg + G);
         unsigned cnt = 0;
         const bool ordered = interval_boundaries(jb.trace, kb, beg, end, [&](unsigned long long, unsigned long long) {
             ++cnt;
         });
         if (!ordered && lane == 0) hr_set_error(&regions[jb.region].error, HR_ERR_ORDER);
-        if (lane == 0) w.counts[i] = cnt;
+        if (lane == 0) counts[i] = cnt;
     }
     __syncthreads();
-    // (c)
-    scan_counts_body(w, total_int, regions);
-    __syncthreads();
-    // (d)
-    const unsigned n_waves = w.ctl->n_waves;
-    for (unsigned q = warp; q < n_need && n_waves; q += blockDim.x >> 5) {
-        const unsigned i = s_list[q];
-        const unsigned long long beg = (unsigned long long)i * G, end = min(n, beg + G);
-        unsigned off = w.counts[i];
-        interval_boundaries(jb.trace, kb, beg, end, [&](unsigned long long p, unsigned long long k) {
-            if (lane == 0 && off < n_waves) {
-                w.wave_start[off] = p;
-                w.wave_key[off] = k;
-            }
-            ++off;
-        });
+    return scan_counts(counts, jb.n_int);
+}
+
+// The boundaries of interval i, from the job's wave `off` on, into the wave table
+// (one warp); `first` is the job's first wave.
+__device__ __forceinline__ void write_interval(const hr_jobd& jb, hr_work& w, unsigned i, unsigned long long first,
+                                               unsigned off)
+{
+    const unsigned long long beg = (unsigned long long)i * jb.G, end = min(jb.n, beg + jb.G);
+    interval_boundaries(jb.trace, jb.kb, beg, end, [&](unsigned long long p, unsigned long long k) {
+        if ((threadIdx.x & 31) == 0 && first + off < w.max_waves) {
+            w.wave_start[first + off] = p;
+            w.wave_key[first + off] = k;
+        }
+        ++off;
+    });
+}
+
+// The whole pre-pass of one trace in one CTA, so that a check costs two launches:
+// the waves, the stages, and the choice of the checker when the caller left that
+// open.
+__global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, hr_work w, hr_region_dev* regions)
+{
+    __shared__ IntervalList s_list;
+    const unsigned warp = threadIdx.x >> 5;
+    const hr_jobd& jb = P.job[0];
+    hr_region_dev& rg = regions[jb.region];
+    const unsigned found = count_waves(jb, w.counts, s_list, regions);
+    unsigned long long waves = found;
+    if (w.cont) waves += rg.group_waves - (key_at(jb.trace, 0, jb.kb) == rg.last_key);  // (a wave cut in two counts once)
+    const bool over = waves > w.max_waves;
+    if (threadIdx.x == 0) {
+        hr_jobd j0 = jb;
+        j0.done_ns = 0;
+        j0.wave_begin = 0;
+        j0.n_waves = over ? 0u : found;
+        w.jobs[0] = j0;
+        w.ctl->n_jobs = 1;
+        w.ctl->t0_ns = globaltimer();
+        reset_ctl(w.ctl, j0.n_waves);
+        if (over) hr_set_error(&rg.error, HR_ERR_CAPACITY);
     }
+    for (unsigned q = warp; q < s_list.n && !over; q += blockDim.x >> 5)
+        write_interval(jb, w, s_list.at[q], 0, w.counts[s_list.at[q]]);
     __syncthreads();
-    // (e)
     stages_one_job(w, regions);
-    // (f)
     if (w.bin.automatic) {
         __syncthreads();
-        bin_choose(w, jb, regions[jb.region], s_list);
+        bin_choose(w, jb, rg, s_list.at);
+    }
+}
+
+// A batch's waves, one CTA per job: their number and the intervals' offsets ...
+__global__ void __launch_bounds__(1024) hr_batch_count(const __grid_constant__ JobParams<HR_MAX_BATCH> P, hr_work w,
+                                                       hr_region_dev* regions)
+{
+    __shared__ IntervalList s_list;
+    const hr_jobd& jb = P.job[blockIdx.x];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        w.ctl->n_jobs = P.n;
+        w.ctl->t0_ns = globaltimer();
+    }
+    const unsigned found = count_waves(jb, w.counts + jb.int_begin, s_list, regions);
+    if (threadIdx.x == 0) {
+        hr_jobd j = jb;
+        j.done_ns = 0;
+        j.n_waves = found;
+        w.jobs[blockIdx.x] = j;
+    }
+}
+
+// ... then their starts and keys, after those of the jobs before.  Measured on 64
+// traces (110M records), both kernels and hr_build_stages: 105 us
+// (213 us with one scan over all jobs' intervals in four launches).
+__global__ void __launch_bounds__(1024) hr_batch_waves(const __grid_constant__ JobParams<HR_MAX_BATCH> P, hr_work w)
+{
+    const hr_jobd& jb = P.job[blockIdx.x];
+    unsigned long long total;
+    block_exclusive_scan(threadIdx.x < blockIdx.x ? w.jobs[threadIdx.x].n_waves : 0u, &total);  // (blockIdx.x < 1024)
+    const unsigned found = w.jobs[blockIdx.x].n_waves;
+    const unsigned* counts = w.counts + jb.int_begin;
+    for (unsigned i = threadIdx.x >> 5; i < jb.n_int; i += blockDim.x >> 5) {
+        const unsigned off = counts[i], next = i + 1 < jb.n_int ? counts[i + 1] : found;
+        if (off != next) write_interval(jb, w, i, total, off);
     }
 }
 
@@ -1188,14 +1119,25 @@ __global__ void hr_sync_kernel(hr_region_dev* region)
     region->used = 1;
 }
 
-__global__ void hr_reset_state(hr_region_dev* region)
+__global__ void hr_reset_state(hr_region_dev* region, unsigned long long* shadow, unsigned long long shadow_bytes)
 {
-    region->n_races = 0;
-    region->error = 0;
-    region->flags = 0;
-    region->last_key = 0;
-    region->used = 0;
-    for (int i = 0; i < 4; ++i) region->counters[i] = 0;
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+        region->n_races = 0;
+        region->error = 0;
+        region->flags = 0;
+        region->last_key = 0;
+        region->used = 0;
+        for (int i = 0; i < 4; ++i) region->counters[i] = 0;
+    }
+    // the shadow, 16 bytes a store, a 4-byte tail
+    unsigned char* p = reinterpret_cast<unsigned char*>(shadow);
+    const unsigned long long step = 16ull * gridDim.x * blockDim.x;
+    for (unsigned long long i = 16ull * (blockIdx.x * blockDim.x + threadIdx.x); i < shadow_bytes; i += step) {
+        if (i + 16 <= shadow_bytes)
+            *reinterpret_cast<ulonglong2*>(p + i) = make_ulonglong2(0ull, 0ull);
+        else
+            for (unsigned long long k = i; k < shadow_bytes; k += 4) *reinterpret_cast<unsigned*>(p + k) = 0u;
+    }
 }
 
 __global__ void hr_reconfigure_state(hr_region_dev* region, unsigned long long n_words, hr_geom geom)
@@ -1261,17 +1203,6 @@ void hr_plan_intervals(unsigned long long n, unsigned budget, unsigned* G, unsig
     *n_int = (unsigned)((n + g - 1) / g);
 }
 
-template <unsigned CAP>
-static void launch_prepass(const JobParams<CAP>& P, unsigned total_int, hr_region_dev* d_regions, const hr_work& w,
-                           cudaStream_t stream)
-{
-    const unsigned blocks = (total_int + 7) / 8 < 4096 ? (total_int + 7) / 8 : 4096;
-    hr_scan_intervals<CAP><<<blocks, 256, 0, stream>>>(P, total_int, w, d_regions);
-    hr_scan_counts<<<1, 1024, 0, stream>>>(w, total_int, d_regions);
-    hr_write_waves<CAP><<<blocks, 256, 0, stream>>>(P, total_int, w);
-    hr_build_stages<<<1, 1024, 0, stream>>>(w, d_regions);
-}
-
 cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const hr_jobd* jobs, unsigned n_jobs,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream,
                            cudaEvent_t before_check, unsigned* launches)
@@ -1289,23 +1220,22 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
     if (n_jobs == 0 || n_jobs > HR_MAX_BATCH || n_jobs > w.max_jobs) return cudaErrorInvalidValue;
     const unsigned total_int = jobs[n_jobs - 1].int_begin + jobs[n_jobs - 1].n_int;
     if (total_int > w.max_intervals) return cudaErrorInvalidValue;
-    unsigned prepass_launches = 4;
+    unsigned prepass_launches = 3;
+    for (unsigned j = 0; j < n_jobs; ++j)
+        if (jobs[j].n_int > HR_SMALL_INTERVALS) return cudaErrorInvalidValue;
     if (n_jobs == 1) {
         JobParams<1> P;
         P.n = 1;
         P.job[0] = jobs[0];
-        if (total_int <= HR_SMALL_INTERVALS) {  // the whole pre-pass in one CTA
-            hr_prepass_small<<<1, 1024, 0, stream>>>(P, total_int, w, d_regions);
-            prepass_launches = 1;
-        } else {
-            if (w.bin.automatic) return cudaErrorInvalidValue;  // the choice is made in the one-CTA pre-pass
-            launch_prepass(P, total_int, d_regions, w, stream);
-        }
+        hr_prepass_single<<<1, 1024, 0, stream>>>(P, w, d_regions);
+        prepass_launches = 1;
     } else {
-        static thread_local JobParams<HR_MAX_BATCH> P;  // 24 KB: off the stack; copied into the launch
+        static thread_local JobParams<HR_MAX_BATCH> P;  // 28 KB: off the stack; copied into the launch
         P.n = n_jobs;
         for (unsigned j = 0; j < n_jobs; ++j) P.job[j] = jobs[j];
-        launch_prepass(P, total_int, d_regions, w, stream);
+        hr_batch_count<<<n_jobs, 1024, 0, stream>>>(P, w, d_regions);
+        hr_batch_waves<<<n_jobs, 1024, 0, stream>>>(P, w);
+        hr_build_stages<<<1, 1024, 0, stream>>>(w, d_regions);
     }
     if (before_check) cudaEventRecord(before_check, stream);
     if (launches) *launches = prepass_launches + 1 + (binned ? 5 : 0);
@@ -1349,8 +1279,14 @@ cudaError_t hr_launch_sync_kernel(hr_region_dev* d_region, cudaStream_t stream)
 cudaError_t hr_launch_reset(hr_region_dev* d_region, unsigned long long* shadow, unsigned long long shadow_bytes,
                             cudaStream_t stream)
 {
-    cudaError_t e = cudaMemsetAsync(shadow, 0, shadow_bytes, stream);
-    if (e != cudaSuccess) return e;
-    hr_reset_state<<<1, 1, 0, stream>>>(d_region);
+    // Up to 4 MB one launch does it all: a memset and a kernel take about 2 us of the
+    // stream and two launches.  The memset is as fast as the memory for larger ones.
+    if (shadow_bytes > HR_RESET_FUSED) {
+        const cudaError_t e = cudaMemsetAsync(shadow, 0, shadow_bytes, stream);
+        if (e != cudaSuccess) return e;
+        shadow_bytes = 0;
+    }
+    const unsigned blocks = (unsigned)((shadow_bytes + 256 * 64 - 1) / (256 * 64));  // 4 stores a thread
+    hr_reset_state<<<blocks ? blocks : 1, 256, 0, stream>>>(d_region, shadow, shadow_bytes);
     return cudaGetLastError();
 }

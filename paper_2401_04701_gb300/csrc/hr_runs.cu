@@ -533,7 +533,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                             done = true;
                             break;
                         }
-                        if (tries >= w.cas_cap) break;
+                        if (tries >= w.cas_cap + ((defer >> k) & 1u)) break;  // (a deferred access has not tried yet)
                         lc_cas++;
                         const unsigned long long x = hr_shadow_cas(shadow, wd, sv, nv, g);
                         if (x == sv) {
