@@ -344,7 +344,10 @@ hr_status hr_destroy(hr_ctx* ctx);
  * of the checker).  Ids 0..5 are shapes of the per-wave checker: a variant
  * fixes the consumer warps per CTA, the records each consumer lane takes per
  * tile and whether lanes on the same word are aggregated; even ids aggregate
- * and the odd id after each is the same shape without aggregation.  Id 6 is the
+ * and the odd id after each is the same shape without aggregation.  Until
+ * hr_set_variant or hr_autotune chooses one (hr_get_variant then says 0), the
+ * library picks the faster checker for each check by its size; races, counts
+ * and shadows are the same with every one.  Id 6 is the
  * binned checker, which hr_variant_desc reports with zero records per lane and
  * zero consumer warps: the accesses are moved into (4096-word shadow segment,
  * wave) buckets and persistent thread groups apply each segment's buckets to a

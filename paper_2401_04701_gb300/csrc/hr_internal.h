@@ -294,6 +294,24 @@ constexpr unsigned HR_N_VARIANTS = HR_N_SHAPES + 1;  // ids a caller may choose
 // Internal id of the checker that also carries the every-epoch path (shape of
 // variant 3); checks on regions in that report mode use it.
 constexpr unsigned HR_EVERY_EPOCH_VARIANT = HR_N_VARIANTS;
+// Batches for which no variant was chosen: four records a lane without aggregation,
+// the fastest shape of every batch measured.  Variants 0, 1, 2, 3: 64 uneven
+// traces (tree reductions and global-memory mixes, 110M records) 3.00, 2.20, 2.72,
+// 2.39 ms; 16 power-law pushes (38M) 2.27, 1.60, 1.68, 1.70 ms.
+constexpr unsigned HR_BATCH_DEFAULT = 1;
+// Single traces for which none was chosen: two records a lane (variant 3) when words
+// are met again and again (the accesses mostly end early, and more warps hide more
+// latency) or the trace is small (its waves then reach more warps), else four
+// (variant 1).  Variants 0, 1, 2, 3: tree reductions of 0.1M, 1M and 10M records
+// 102, 72, 75, 53 us, 124, 94, 105, 79 us and 237, 199, 215, 182 us; power-law pushes
+// of 2.6M, 20M and 67M records 175, 173, 165, 173 us, 576, 550, 489, 475 us and
+// 1148, 1073, 953, 910 us; global-memory traces of 0.29M, 4.7M and 75M records
+// (variants 0, 1, 3) 289, 247, 218 us, 362, 331, 390 us and 2145, 1861, 2015 us.
+constexpr unsigned long long HR_SMALL_TRACE = 1ull << 19;
+constexpr unsigned hr_default_variant(unsigned long long n, unsigned long long n_words)
+{
+    return n / 8 >= n_words || n < HR_SMALL_TRACE ? 3u : 1u;
+}
 constexpr unsigned hr_variant_consumers(unsigned v)
 {
     return v == HR_EVERY_EPOCH_VARIANT ? 8u
