@@ -47,6 +47,16 @@ inline hr_geom hr_desc_geom(const hr_region_desc& d)
     return hr_make_geom(d.block_dim, d.warp_size, d.shadow_bytes == 4 ? 4u : 8u, hr_desc_tid_bits(d), d.report_mode);
 }
 
+// What hr_report and hr_counters tell of a region, kept in page-locked host memory
+// that the device writes: by the last CTA of every check and by every reset, so a
+// report needs no copy once the region's work is done.  (A region with a device
+// view is read from the device: instrumented kernels write its state themselves.)
+struct hr_told {
+    unsigned long long n_races;
+    unsigned long long counters[4];
+    unsigned int error, flags;
+};
+
 // Per-region state in device memory.
 struct hr_region_dev {
     unsigned long long* shadow;   // n_words shadow values
@@ -64,6 +74,7 @@ struct hr_region_dev {
     unsigned long long counters[4];  // accesses, CAS attempts, CAS retries, accesses without a shadow access
     hr_geom geom;
     hr_filter filter;             // monitored words, blocks, lanes (hr_set_filter)
+    hr_told* told;                // the host's copy of the report (NULL: none)
 };
 
 // the filter that monitors every access
@@ -116,7 +127,7 @@ struct hr_ctl {
     unsigned n_stages;
     unsigned total_items;
     unsigned n_jobs;
-    unsigned n_intervals;
+    unsigned exited;       // CTAs of the check's last kernel that are done
     unsigned binned;       // 1: the binned checker took this check (the per-wave checker then has no items)
     unsigned long long t0_ns;  // device clock when the check's first kernel started
     unsigned bin_parts;    // binned checker: (slice, wave) parts of the trace

@@ -92,6 +92,7 @@ __device__ unsigned scan_counts(unsigned* counts, unsigned n_int)
 __device__ void reset_ctl(hr_ctl* c, unsigned n_waves)
 {
     c->ticket = 0;
+    c->exited = 0;
     c->abort = 0;
     c->total_items = 0;
     c->n_stages = 0;
@@ -1109,6 +1110,8 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
         publish(it, t_stage);
     }
     flush();
+    tell_when_last(w, regions, HR_CONSUMERS * 32,
+                   [] { asm volatile("bar.sync 1, %0;" ::"n"(HR_CONSUMERS * 32) : "memory"); });
 }
 
 __global__ void hr_sync_kernel(hr_region_dev* region)
@@ -1128,6 +1131,7 @@ __global__ void hr_reset_state(hr_region_dev* region, unsigned long long* shadow
         region->last_key = 0;
         region->used = 0;
         for (int i = 0; i < 4; ++i) region->counters[i] = 0;
+        if (region->told) *region->told = hr_told{};
     }
     // the shadow, 16 bytes a store, a 4-byte tail
     unsigned char* p = reinterpret_cast<unsigned char*>(shadow);
