@@ -171,9 +171,12 @@ __device__ void stages_one_job(hr_work& w, hr_region_dev* regions)
         w.ctl->n_stages = n_st;
         w.ctl->total_items = failed ? 0u : (unsigned)tot;
         // a zero shadow (new or reset region), one cleared before the first wave
-        // (used == 2), or one last written by an older kernel: nothing in it is live
+        // (used == 2), or one last written by an older kernel: nothing in it is live.
+        // (The automatic route keeps such an older kernel's values where the per-wave
+        // checker would: it reads them.)
         w.ctl->fresh = !failed && nw > 0 && !w.views &&
-                       (rg.used != 1 || (w.wave_key[jb.wave_begin] >> 32) > (rg.last_key >> 32));
+                       (rg.used != 1 ||
+                        (!w.bin.automatic && (w.wave_key[jb.wave_begin] >> 32) > (rg.last_key >> 32)));
         if (!failed && nw > 0) {
             rg.group_waves = nw + (w.cont ? rg.group_waves - (w.wave_key[jb.wave_begin] == rg.last_key) : 0ull);
             rg.last_key = w.wave_key[jb.wave_begin + nw - 1];

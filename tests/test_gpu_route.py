@@ -39,7 +39,7 @@ def trace_of(seed, n=N, words=WORDS, waves=30, kernels=1, threads=1 << 14, hot=0
     return r
 
 
-# name -> (trace arguments, region arguments, filter, calls)
+# name -> (trace arguments, region arguments, filter, calls (0: one per kernel))
 CASES = {
     "taken": (dict(), dict(), {}, 1),
     "block of 96": (dict(), dict(block_dim=96), {}, 1),
@@ -48,6 +48,7 @@ CASES = {
     "hub word": (dict(hot=0.4), dict(), {}, 1),
     "kernels, clears": (dict(waves=3, kernels=17), dict(), {}, 1),
     "three calls": (dict(waves=60, n=3 * N), dict(), {}, 3),
+    "a call per kernel": (dict(waves=20, kernels=3, n=3 * N), dict(), {}, 0),
     "compact": (dict(waves=9), dict(shadow_bytes=4, tid_bits=14), {}, 1),
     "wide tids": (dict(tid_base=1 << 22), dict(), {}, 1),
     "window": (dict(words=2 * WORDS), dict(), dict(word_lo=1000, word_hi=1000 + WORDS), 1),
@@ -59,7 +60,9 @@ CASES = {
 def check(hr, trace, reg, filt, calls, variant, capture=False):
     import torch
     d = torch.from_numpy(trace.view(np.uint8)).cuda()
-    cuts = [16 * (len(trace) * i // calls) for i in range(calls)] + [d.numel()]
+    cuts = [16 * (len(trace) * i // calls) for i in range(calls)] if calls else \
+        [16 * int(i) for i in np.unique(trace["kernel"], return_index=True)[1]]
+    cuts.append(d.numel())
     shadow = torch.full((reg["n_words"],), -1, dtype=torch.int64, device="cuda")
     with hr.Checker([reg], report_capacity=1 << 20, buffers=[shadow]) as ck:
         if filt:
@@ -88,7 +91,8 @@ def test_default_equals_per_wave(hr, name):
     want = check(hr, trace, reg, filt, calls, 3)
     assert want[0] == hr.HR_OK and want[1] == len(want[2]) > 100
     assert check(hr, trace, reg, filt, calls, None) == want
-    assert check(hr, trace, reg, filt, calls, hr.binned_variant()) == want
+    got = check(hr, trace, reg, filt, calls, hr.binned_variant())
+    assert got[:3] == want[:3] and (calls == 0 or got == want)   # (0: drops an older kernel's values)
 
 
 def test_capture(hr):
