@@ -95,10 +95,11 @@ def test_default_equals_per_wave(hr, name):
     assert got[:3] == want[:3] and (calls == 0 or got == want)   # (0: drops an older kernel's values)
 
 
-def test_capture(hr):
+@pytest.mark.parametrize("variant", [None, 3, 5, 6])
+def test_capture(hr, variant):
     trace = trace_of(5)
     reg = dict(n_words=WORDS, block_dim=64)
-    assert check(hr, trace, reg, {}, 1, None, capture=True) == check(hr, trace, reg, {}, 1, 3)
+    assert check(hr, trace, reg, {}, 1, variant, capture=True) == check(hr, trace, reg, {}, 1, 3)
 
 
 @pytest.mark.parametrize("what", ["order", "range", "unsupported"])
