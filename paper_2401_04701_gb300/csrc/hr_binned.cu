@@ -634,34 +634,40 @@ __device__ __forceinline__ void group_sync(unsigned id, unsigned n)
     asm volatile("bar.sync %0, %1;" ::"r"(id), "r"(n) : "memory");
 }
 
-// working value (4 bytes) <-> 8-byte layout, tid in tb bits
-__device__ __forceinline__ unsigned long long pg_expand(unsigned x, const hr_geom& gw) { return hr_expand32(x, gw); }
-__device__ __forceinline__ unsigned pg_compress(unsigned long long v, const hr_geom& gw) { return hr_compress64(v, gw); }
-
 // The FSM step of Algorithm 1 on the 4-byte working form (the compact storage
-// form with tid width tb, hr_expand32): the same transition as
-// hr_fsm_step_pow2 on the expanded value, with 32-bit operations only.  wbits
+// form with tid width tb, hr_expand32): the same transition as hr_fsm_step
+// (POW2: hr_fsm_step_pow2) on the expanded value, without expanding it (blocks of 96
+// threads, 8.3M records: hr_bin_groups 102 -> 80 us).  wbits
 // is the wave's kernel tag, bc and wc placed where the form keeps them; mbc and
 // mwc mask the bc and wc fields; keep_w and keep_b keep the tid bits of a
 // warp's and of a block's first thread (~(warp_size - 1), ~(block_dim - 1)).
+template <bool POW2>
 __device__ __forceinline__ unsigned compact_step(unsigned x, unsigned tid, unsigned op, unsigned wbits, unsigned mbc,
-                                                 unsigned mwc, unsigned tidmask, unsigned bd_shift,
-                                                 unsigned ws_shift, unsigned keep_w, unsigned keep_b,
-                                                 const unsigned char* tab, unsigned* raced)
+                                                 unsigned mwc, unsigned tidmask, const hr_geom& g, unsigned keep_w,
+                                                 unsigned keep_b, const unsigned char* tab, unsigned* raced)
 {
     const unsigned d = x ^ wbits;
     unsigned os = x >> 27;
     if (d & 0x07000000u) os = HR_STATE_INIT;  // another kernel's value (or INIT already)
     const unsigned xt = (x & tidmask) ^ tid;
-    const unsigned trel = xt == 0u ? HR_TREL_SAME : (xt >> bd_shift) ? HR_TREL_GRID
-                        : (xt >> ws_shift) ? HR_TREL_BLOCK : HR_TREL_WARP;
+    const unsigned trel = !POW2 ? hr_thread_rel(tid, x & tidmask, g)
+                        : xt == 0u ? HR_TREL_SAME : (xt >> g.bd_shift) ? HR_TREL_GRID
+                        : (xt >> g.ws_shift) ? HR_TREL_BLOCK : HR_TREL_WARP;
     const unsigned srel = (d & mbc) ? HR_SREL_BLOCK : ((d & mwc) ? HR_SREL_WARP : HR_SREL_UNSYNC);
     const unsigned e = tab[(os << 6) | (op << 4) | (trel << 2) | srel];
     const unsigned ns = e & 31u, lvl = e >> 5;
     unsigned nx = (ns << 27) | (wbits & 0x07000000u);
-    if (lvl >= HR_LVL_THREAD && lvl <= HR_LVL_BLOCK)
-        nx |= (tid & (lvl == HR_LVL_THREAD ? ~0u : (lvl == HR_LVL_WARP ? keep_w : keep_b))) |
-              (wbits & (lvl == HR_LVL_BLOCK ? mbc : (mbc | mwc)));
+    if (lvl >= HR_LVL_THREAD && lvl <= HR_LVL_BLOCK) {
+        unsigned who = tid;
+        if (POW2) {
+            who &= lvl == HR_LVL_THREAD ? ~0u : (lvl == HR_LVL_WARP ? keep_w : keep_b);
+        } else if (lvl != HR_LVL_THREAD) {
+            unsigned wh, bh;
+            hr_scope_heads(tid, g, &wh, &bh);
+            who = lvl == HR_LVL_WARP ? wh : bh;
+        }
+        nx |= who | (wbits & (lvl == HR_LVL_BLOCK ? mbc : (mbc | mwc)));
+    }
     if (ns == HR_STATE_RACE && os != HR_STATE_RACE) *raced = 1u + os;
     return nx;
 }
@@ -788,23 +794,15 @@ __device__ __forceinline__ void pg_run(unsigned char* gbase, PCommon& C, const h
                         op = (r.y >> 16) & 0xFFu;
                         tid = r.x;
                     }
-                    auto as64 = [&](auto v) -> unsigned long long {
-                        if constexpr (COMPACT) return pg_expand((unsigned)v, gw);
-                        else return (unsigned long long)v;
-                    };
                     // one FSM step from a stored value to the value to store
                     auto step = [&](auto stored, unsigned* raced) -> decltype(stored) {
-                        if constexpr (COMPACT && POW2) {
-                            return compact_step(stored, tid, op, wbits, mbc, mwc, tidmask, g.bd_shift, g.ws_shift,
-                                                keep_w, keep_b, C.tab, raced);
-                        } else {
-                            const unsigned long long o = as64(stored);
-                            const unsigned long long nv =
-                                POW2 ? hr_fsm_step_pow2(o, tid, op, bc, wc, ktag, g.bd_shift, g.ws_shift, C.tab, raced)
-                                     : hr_fsm_step(o, tid, op, bc, wc, ktag, g, C.tab, raced);
-                            if constexpr (COMPACT) return pg_compress(nv, gw);
-                            else return nv;
-                        }
+                        if constexpr (COMPACT)
+                            return compact_step<POW2>(stored, tid, op, wbits, mbc, mwc, tidmask, g, keep_w, keep_b, C.tab,
+                                                      raced);
+                        else
+                            return POW2 ? hr_fsm_step_pow2(stored, tid, op, bc, wc, ktag, g.bd_shift, g.ws_shift, C.tab,
+                                                           raced)
+                                        : hr_fsm_step(stored, tid, op, bc, wc, ktag, g, C.tab, raced);
                     };
                     auto stored = G.sh[wis];
                     unsigned raced = 0;
