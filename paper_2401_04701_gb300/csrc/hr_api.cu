@@ -1,6 +1,7 @@
 // hr_api.cu - the C-ABI entry points declared in include/hirace.h.
 #include <cuda_runtime.h>
 
+#include <cstddef>
 #include <cstdlib>
 #include <cstring>
 #include <new>
@@ -12,6 +13,11 @@ namespace {
 
 // the Python binding mirrors these layouts (paper_2401_04701_gb300/hirace.py)
 static_assert(sizeof(hr_filter) == 48 && sizeof(hr_view) == 168, "hr_filter / hr_view layouts");
+// a region's state holds what is told of it in one piece
+static_assert(offsetof(hr_told, counters) == offsetof(hr_region_dev, counters) - offsetof(hr_region_dev, n_races) &&
+                  offsetof(hr_told, error) == offsetof(hr_region_dev, error) - offsetof(hr_region_dev, n_races) &&
+                  offsetof(hr_told, flags) == offsetof(hr_region_dev, flags) - offsetof(hr_region_dev, n_races),
+              "hr_told layout");
 
 struct RegionHost {
     hr_region_desc desc{};
@@ -595,17 +601,11 @@ static hr_status fetch_told(hr_ctx* ctx, uint32_t region, hr_told* out)
     RegionHost& r = ctx->regions[region];
     cudaError_t e = r.captured ? cudaDeviceSynchronize() : cudaEventSynchronize(r.done);
     if (e != cudaSuccess) return cuda_status(e);
-    if (!r.views) {
-        memcpy(out, ctx->told + region, sizeof *out);
-        return HR_OK;
+    if (r.views) {
+        e = cudaMemcpyAsync(ctx->told + region, &r.d->n_races, sizeof *out, cudaMemcpyDeviceToHost, ctx->copies);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->copies);
     }
-    hr_region_dev h;
-    e = cudaMemcpyAsync(&h, r.d, sizeof h, cudaMemcpyDeviceToHost, ctx->copies);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->copies);
-    out->n_races = h.n_races;
-    for (int i = 0; i < 4; ++i) out->counters[i] = h.counters[i];
-    out->error = h.error;
-    out->flags = h.flags;
+    memcpy(out, ctx->told + region, sizeof *out);
     return cuda_status(e);
 }
 

@@ -63,7 +63,9 @@ struct hr_region_dev {
     hr_race* ring;                // ring_cap race records
     unsigned long long n_words;
     unsigned long long ring_cap;
+    // (an hr_told, which hr_report copies from a region with a device view)
     unsigned long long n_races;   // races found (may exceed ring_cap)
+    unsigned long long counters[4];  // accesses, CAS attempts, CAS retries, accesses without a shadow access
     unsigned int error;           // sticky first error (hr_status)
     unsigned int flags;           // HR_FLAG_* bits
     unsigned long long group_waves;  // waves of the record group a host-memory check is in (hr_work::cont)
@@ -71,7 +73,6 @@ struct hr_region_dev {
     unsigned int used;            // 1: a record was processed since init/reset; 2: the shadow's
                                   // contents are unknown (cleared before the first wave)
     unsigned int region;
-    unsigned long long counters[4];  // accesses, CAS attempts, CAS retries, accesses without a shadow access
     hr_geom geom;
     hr_filter filter;             // monitored words, blocks, lanes (hr_set_filter)
     hr_told* told;                // the host's copy of the report (NULL: none)
