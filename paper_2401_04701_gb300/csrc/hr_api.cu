@@ -373,6 +373,7 @@ static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_t
     w.test_flags = ctx->test_flags;
     w.views = r.views ? 1u : 0u;
     w.cont = cont ? 1u : 0u;
+    w.tell = 1u;
     unsigned variant = ctx->chosen ? ctx->variant : hr_default_variant(n, r.desc.n_words);
     if (!aggregate && variant < HR_N_SHAPES) variant |= 1u;  // odd ids do not aggregate (nor does the binned one)
     if (r.desc.report_mode == HR_REPORT_EVERY_EPOCH) variant = HR_EVERY_EPOCH_VARIANT;
@@ -557,6 +558,7 @@ extern "C" hr_status hr_check_batch(hr_ctx* ctx, const hr_job* jobs, uint32_t n_
     if (ctx->profile) pc = take_events(ctx);
     if (ctx->profile) cudaEventRecord(pc.begin, s);
     hr_work w = ctx->batch;
+    w.tell = 1u;
     w.wait_ns = ctx->wait_ns;
     w.cas_cap = ctx->cas_cap;
     unsigned variant = ctx->variant == HR_BIN_VARIANT ? HR_BIN_FALLBACK : ctx->variant;  // not for batches

@@ -31,32 +31,6 @@ __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// The end of a check's last kernel, for every CTA of it: the last one writes the
-// jobs' reports to the host's copies.  Called by the CTA's n threads with no shadow,
-// ring or counter update left to do; sync is a barrier of them.
-template <class Sync>
-__device__ __forceinline__ void tell_when_last(const hr_work& w, hr_region_dev* regions, unsigned n, Sync sync)
-{
-    __shared__ unsigned s_is_last;
-    sync();
-    if (threadIdx.x == 0) {
-        __threadfence();
-        s_is_last = atomicAdd(&w.ctl->exited, 1u) + 1u == gridDim.x;
-        __threadfence();
-    }
-    sync();
-    if (!s_is_last) return;
-    for (unsigned j = threadIdx.x; j < w.ctl->n_jobs; j += n) {
-        const volatile hr_region_dev& rg = regions[w.jobs[j].region];
-        hr_told* t = regions[w.jobs[j].region].told;
-        if (!t) continue;
-        t->n_races = rg.n_races;
-        for (int i = 0; i < 4; ++i) t->counters[i] = rg.counters[i];
-        t->error = rg.error;
-        t->flags = rg.flags;
-    }
-}
-
 // Every-epoch mode for a lane's RPL accesses at once (bit k of `act`: slot k
 // holds one): the steps of hr_ep_apply, each over every slot before the next,
 // so each step costs one round trip for all of them and one fence serves them

@@ -48,7 +48,7 @@ inline hr_geom hr_desc_geom(const hr_region_desc& d)
 }
 
 // What hr_report and hr_counters tell of a region, kept in page-locked host memory
-// that the device writes: by the last CTA of every check and by every reset, so a
+// that the device writes: at the end of every check and in every reset, so a
 // report needs no copy once the region's work is done.  (A region with a device
 // view is read from the device: instrumented kernels write its state themselves.)
 struct hr_told {
@@ -75,7 +75,7 @@ struct hr_region_dev {
     unsigned int region;
     hr_geom geom;
     hr_filter filter;             // monitored words, blocks, lanes (hr_set_filter)
-    hr_told* told;                // the host's copy of the report (NULL: none)
+    hr_told* told;                // the host's copy of the report
 };
 
 // the filter that monitors every access
@@ -128,7 +128,7 @@ struct hr_ctl {
     unsigned n_stages;
     unsigned total_items;
     unsigned n_jobs;
-    unsigned exited;       // CTAs of the check's last kernel that are done
+    unsigned n_intervals;
     unsigned binned;       // 1: the binned checker took this check (the per-wave checker then has no items)
     unsigned long long t0_ns;  // device clock when the check's first kernel started
     unsigned bin_parts;    // binned checker: (slice, wave) parts of the trace
@@ -242,6 +242,7 @@ struct hr_work {
     unsigned test_flags;             // HR_TEST_* hooks (tests only)
     unsigned views;                  // 1: a device view of the checked region exists (inline writes may
                                      // carry kernel ordinals the region's last key does not know)
+    unsigned tell;                   // 1: the regions have hr_told copies
     unsigned cont;                   // 1: goes on with the record group of the region's last check, whose
                                      // waves count together against max_waves (single-trace checks only)
     hr_bin bin;                      // binned checker scratch (variant HR_BIN_VARIANT and the automatic route)
@@ -367,8 +368,8 @@ constexpr unsigned long long HR_KEY_MASK = 0xFFFFFFFFFFFFull;
 // kernel launch helpers (hr_kernels.cu)
 // Check n_jobs jobs (1..HR_MAX_BATCH) on the regions of d_regions with the
 // scratch w.  Jobs must name distinct regions and hold n > 0 records.
-// *launches (if not NULL) receives the kernels launched: 2 for a single trace
-// (7 with the binned checker), 4 for a batch.
+// *launches (if not NULL) receives the kernels launched: 3 for a single trace
+// (8 with the binned checker), 5 for a batch; one fewer without w.tell.
 cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w, const hr_jobd* jobs, unsigned n_jobs,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream,
                            cudaEvent_t before_check, unsigned* launches = nullptr);

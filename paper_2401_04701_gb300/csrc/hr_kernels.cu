@@ -92,7 +92,6 @@ __device__ unsigned scan_counts(unsigned* counts, unsigned n_int)
 __device__ void reset_ctl(hr_ctl* c, unsigned n_waves)
 {
     c->ticket = 0;
-    c->exited = 0;
     c->abort = 0;
     c->total_items = 0;
     c->n_stages = 0;
@@ -361,15 +360,22 @@ static_assert(HR_BIN_SAMPLES <= HR_SMALL_INTERVALS, "the sample's counters fit t
 // CTA: (a) the intervals holding a wave boundary (one lane per interval, two keys
 // each) go to the list, (b) a warp per listed interval counts its boundaries,
 // (c) the counts become offsets.  counts: the job's; returns its waves.
+// A boundary found while counting is kept if there is room, so that writing the wave
+// table need not search again (16.0 -> 14.5 us for the pre-pass of a 32-wave trace).
+constexpr unsigned FOUND = 512;
 struct IntervalList {
     unsigned at[HR_SMALL_INTERVALS], n;
+    unsigned n_found;  // boundaries; more than FOUND: not all of them are kept
+    unsigned long long pos[FOUND], key[FOUND];
+    unsigned interval[FOUND], nth[FOUND];
 };
 __device__ unsigned count_waves(const hr_jobd& jb, unsigned* counts, IntervalList& list, hr_region_dev* regions)
 {
     const unsigned lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const unsigned long long n = jb.n, kb = jb.kb, G = jb.G;
-    if (threadIdx.x == 0) list.n = 0;
+    if (threadIdx.x == 0) list.n = list.n_found = 0;
     __syncthreads();
+#pragma unroll 4
     for (unsigned i = threadIdx.x; i < jb.n_int; i += blockDim.x) {
         const unsigned long long beg = (unsigned long long)i * G, end = min(n, beg + G);
         if (i == 0 || key_at(jb.trace, beg - 1, kb) != key_at(jb.trace, end - 1, kb))
@@ -382,7 +388,16 @@ __device__ unsigned count_waves(const hr_jobd& jb, unsigned* counts, IntervalLis
         const unsigned i = list.at[q];
         const unsigned long long beg = (unsigned long long)i * G, end = min(n, beg + G);
         unsigned cnt = 0;
-        const bool ordered = interval_boundaries(jb.trace, kb, beg, end, [&](unsigned long long, unsigned long long) {
+        const bool ordered = interval_boundaries(jb.trace, kb, beg, end, [&](unsigned long long p, unsigned long long k) {
+            if (lane == 0) {
+                const unsigned f = atomicAdd(&list.n_found, 1u);
+                if (f < FOUND) {
+                    list.pos[f] = p;
+                    list.key[f] = k;
+                    list.interval[f] = i;
+                    list.nth[f] = cnt;
+                }
+            }
             ++cnt;
         });
         if (!ordered && lane == 0) hr_set_error(&regions[jb.region].error, HR_ERR_ORDER);
@@ -419,7 +434,7 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
     const unsigned found = count_waves(jb, w.counts, s_list, regions);
     unsigned long long waves = found;
     if (w.cont) waves += rg.group_waves - (key_at(jb.trace, 0, jb.kb) == rg.last_key);  // (a wave cut in two counts once)
-    const bool over = waves > w.max_waves;
+    const bool over = waves > w.max_waves || found > w.max_waves;
     if (threadIdx.x == 0) {
         hr_jobd j0 = jb;
         j0.done_ns = 0;
@@ -431,8 +446,16 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
         reset_ctl(w.ctl, j0.n_waves);
         if (over) hr_set_error(&rg.error, HR_ERR_CAPACITY);
     }
-    for (unsigned q = warp; q < s_list.n && !over; q += blockDim.x >> 5)
-        write_interval(jb, w, s_list.at[q], 0, w.counts[s_list.at[q]]);
+    if (!over && s_list.n_found <= FOUND) {
+        for (unsigned f = threadIdx.x; f < s_list.n_found; f += blockDim.x) {
+            const unsigned at = w.counts[s_list.interval[f]] + s_list.nth[f];
+            w.wave_start[at] = s_list.pos[f];  // (at < found <= max_waves)
+            w.wave_key[at] = s_list.key[f];
+        }
+    } else if (!over) {
+        for (unsigned q = warp; q < s_list.n; q += blockDim.x >> 5)
+            write_interval(jb, w, s_list.at[q], 0, w.counts[s_list.at[q]]);
+    }
     __syncthreads();
     stages_one_job(w, regions);
     if (w.bin.automatic) {
@@ -1113,8 +1136,22 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
         publish(it, t_stage);
     }
     flush();
-    tell_when_last(w, regions, HR_CONSUMERS * 32,
-                   [] { asm volatile("bar.sync 1, %0;" ::"n"(HR_CONSUMERS * 32) : "memory"); });
+}
+
+// The jobs' reports to the host's copies, after a check.  A launch of its own (about
+// 3 us): at the end of the checkers it cost their main loops registers (power-law
+// push of 2^22 vertices 4.54 -> 4.85 ms, tree reduction of 1M records 77 -> 88 us).
+__global__ void hr_tell(const hr_region_dev* regions, const hr_jobd* jobs, const hr_ctl* ctl)
+{
+    for (unsigned j = threadIdx.x; j < ctl->n_jobs; j += blockDim.x) {
+        const hr_region_dev& rg = regions[jobs[j].region];
+        hr_told t;
+        t.n_races = rg.n_races;
+        for (int i = 0; i < 4; ++i) t.counters[i] = rg.counters[i];
+        t.error = rg.error;
+        t.flags = rg.flags;
+        *rg.told = t;
+    }
 }
 
 __global__ void hr_sync_kernel(hr_region_dev* region)
@@ -1134,7 +1171,7 @@ __global__ void hr_reset_state(hr_region_dev* region, unsigned long long* shadow
         region->last_key = 0;
         region->used = 0;
         for (int i = 0; i < 4; ++i) region->counters[i] = 0;
-        if (region->told) *region->told = hr_told{};
+        *region->told = hr_told{};
     }
     // the shadow, 16 bytes a store, a 4-byte tail
     unsigned char* p = reinterpret_cast<unsigned char*>(shadow);
@@ -1210,6 +1247,12 @@ void hr_plan_intervals(unsigned long long n, unsigned budget, unsigned* G, unsig
     *n_int = (unsigned)((n + g - 1) / g);
 }
 
+static cudaError_t launch_tell(hr_region_dev* d_regions, const hr_work& w, unsigned n_jobs, cudaStream_t stream)
+{
+    if (w.tell) hr_tell<<<1, n_jobs < 32 ? 32 : 256, 0, stream>>>(d_regions, w.jobs, w.ctl);
+    return cudaGetLastError();
+}
+
 cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const hr_jobd* jobs, unsigned n_jobs,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream,
                            cudaEvent_t before_check, unsigned* launches)
@@ -1245,12 +1288,15 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
         hr_build_stages<<<1, 1024, 0, stream>>>(w, d_regions);
     }
     if (before_check) cudaEventRecord(before_check, stream);
-    if (launches) *launches = prepass_launches + 1 + (binned ? 5 : 0);
+    if (launches) *launches = prepass_launches + 1 + (binned ? 5 : 0) + (w.tell ? 1 : 0);
     if (binned) {
         const cudaError_t e = hr_launch_binned(d_regions, w, d_table, stream);
         if (e != cudaSuccess) return e;
     }
-    if (runs) return hr_launch_runs(d_regions, w, jobs[0].n, d_table, variant, stream);
+    if (runs) {
+        const cudaError_t e = hr_launch_runs(d_regions, w, jobs[0].n, d_table, variant, stream);
+        return e != cudaSuccess ? e : launch_tell(d_regions, w, n_jobs, stream);
+    }
     const int grid = hr_check_grid_size(variant);
     switch (variant) {
     case 0: launch_variant<true, 4, 8>(grid, d_regions, w, d_table, stream); break;
@@ -1261,7 +1307,7 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
     case 5: launch_variant<false, 1, 8>(grid, d_regions, w, d_table, stream); break;
     default: launch_variant<false, 2, 8, true>(grid, d_regions, w, d_table, stream); break;
     }
-    return cudaGetLastError();
+    return launch_tell(d_regions, w, n_jobs, stream);
 }
 
 cudaError_t hr_launch_reconfigure(hr_region_dev* d_region, unsigned long long n_words, hr_geom geom,

@@ -227,10 +227,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
 
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->total_items;  // binned: the work is done already
-    if (total == 0) {
-        tell_when_last(w, regions, CHECK_THREADS, [] { __syncthreads(); });
-        return;
-    }
+    if (total == 0) return;
     // items per claim: enough to keep the ticket counter out of the way, few
     // enough that a stage's items spread over all warps
     const unsigned claim =
@@ -680,7 +677,6 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
     }
     publish();
     flush();
-    tell_when_last(w, regions, CHECK_THREADS, [] { __syncthreads(); });
 }
 
 template <bool AGG, int RPL, bool EVERY>
