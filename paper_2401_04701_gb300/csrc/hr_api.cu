@@ -305,6 +305,7 @@ static hr_status ensure_bin(RegionHost& r, uint64_t n, cudaStream_t s)
         r.bin.out_cap = n;
     }
     r.bin.n_seg = n_seg;
+    r.bin.every = r.desc.report_mode == HR_REPORT_EVERY_EPOCH ? 1u : 0u;
     r.bin.pow2 = hr_desc_geom(r.desc).bd_shift != ~0u ? 1u : 0u;
     return HR_OK;
 }
@@ -319,7 +320,8 @@ static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
 {
     const unsigned cap_seg = (unsigned)((r.capacity + HR_BIN_SEG - 1) / HR_BIN_SEG);
     const uint64_t n_seg = (r.desc.n_words + HR_BIN_SEG - 1) / HR_BIN_SEG;
-    if (ctx->chosen || r.desc.report_mode == HR_REPORT_EVERY_EPOCH || n < HR_BIN_AUTO_MIN_N || n > HR_BIN_AUTO_MAX_N ||
+    const bool every = r.desc.report_mode == HR_REPORT_EVERY_EPOCH;  // (the variant does not apply to them)
+    if ((ctx->chosen && !every) || n < HR_BIN_AUTO_MIN_N || n > HR_BIN_AUTO_MAX_N ||
         n_seg < HR_BIN_AUTO_SEGS || cap_seg > HR_BIN_MAX_SEGS || ctx->test_flags || ctx->cas_cap < HR_DEFAULT_CAS_CAP)
         return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;

@@ -144,6 +144,7 @@ struct hr_ctl {
     unsigned bin_max_seg;  // binned checker: accesses of the fullest segment
     unsigned bin_count;    // binned checker: accesses counted into buckets
     unsigned bin_skip;     // automatic route: 1: the pre-pass left this check to the per-wave checker
+    unsigned bin_every;    // 1: every-epoch region (binned only in the 4-byte working form)
     unsigned bin_err;      // automatic route: 1: the count pass met an error (the per-wave checker then
                            // does the check, and reports it)
 };
@@ -155,7 +156,7 @@ struct hr_ctl {
 // binned kernels).  Read by the kernels after the count and scan passes.
 __host__ __device__ inline bool hr_bin_taken(const hr_ctl* c)
 {
-    return c->binned && !c->bin_err && !(c->bin_count >= HR_BIN_SKEW_MIN && (unsigned long long)c->bin_max_seg * HR_BIN_SKEW > c->bin_count);
+    return c->binned && !c->bin_err && !(c->bin_every && !c->bin_tbits) && !(c->bin_count >= HR_BIN_SKEW_MIN && (unsigned long long)c->bin_max_seg * HR_BIN_SKEW > c->bin_count);
 }
 
 // The automatic route: a check for which no variant was chosen takes the binned
@@ -172,6 +173,9 @@ __host__ __device__ inline bool hr_bin_taken(const hr_ctl* c)
 // 2^26 words 95 / 267.  A check that the pre-pass leaves to the per-wave checker
 // pays about 20 us for the binned kernels that find nothing to do; that counts on the
 // per-wave checker's side, and smaller checks and regions never get there.
+// Every-epoch regions take it when nothing in their shadow is live: there the
+// per-wave checker needs 40 ps a record and the binned one 30 ps (pre-pass and check,
+// 32 waves: 4.7M records 565 and 245 us, 18.8M 1043 and about 620 us).
 constexpr unsigned long long HR_BIN_AUTO_MIN_N = 1ull << 18;     // records
 constexpr unsigned long long HR_BIN_AUTO_MAX_N = 1ull << 27;     // (1 GiB of bucketed accesses)
 constexpr unsigned long long HR_BIN_AUTO_BYTES = 3ull << 30;     // scratch a context allocates for it, at most
@@ -180,7 +184,8 @@ constexpr unsigned HR_BIN_SAMPLES = 4096;                        // records samp
 constexpr unsigned long long HR_BIN_AUTO_PS_WAVE = 9000000, HR_BIN_AUTO_PS_REC = 28, HR_BIN_AUTO_PS_SKIP = 20000000,
                              HR_BIN_AUTO_PS_BIN = 75000000,
                              HR_BIN_AUTO_PS_BIN_REC = 18, HR_BIN_AUTO_PS_BIN_5_WORDS = 12,
-                             HR_BIN_AUTO_PS_BIN_FULLEST = 1600;
+                             HR_BIN_AUTO_PS_BIN_FULLEST = 1600, HR_BIN_AUTO_PS_REC_EVERY = 40,
+                             HR_BIN_AUTO_PS_BIN_REC_EVERY = 30, HR_BIN_AUTO_PS_BIN_FULLEST_EVERY = 4000;
 
 // Scratch of the binned checker (hr_binned.cu), one per region.  The region's
 // shadow is cut into segments of HR_BIN_SEG words.  The trace is cut into one
@@ -217,6 +222,7 @@ struct hr_bin {
     unsigned clusters;       // scatter clusters
     unsigned sub;            // count slices per cluster slice
     unsigned slices;         // count slices (CTAs of the count pass): clusters * sub
+    unsigned every;          // 1: the region reports every epoch
     unsigned automatic;      // 1: no variant was chosen; the check takes this route where it is faster
     unsigned pow2;           // 1: block size and warp size are powers of two (bit-operation FSM step)
 };

@@ -102,6 +102,8 @@ __device__ void reset_ctl(hr_ctl* c, unsigned n_waves)
     c->bin_count = 0;
     c->bin_skip = 0;
     c->bin_err = 0;
+    c->bin_every = 0;
+    c->bin_tbits = 0;
     c->n_waves = n_waves;
 }
 
@@ -321,10 +323,11 @@ __device__ void bin_choose(hr_work& w, const hr_jobd& jb, const hr_region_dev& r
 {
     const unsigned waves = w.ctl->n_waves;
     const unsigned long long per_wave =
-        HR_BIN_AUTO_PS_SKIP + waves * HR_BIN_AUTO_PS_WAVE + jb.n * HR_BIN_AUTO_PS_REC;
+        HR_BIN_AUTO_PS_SKIP + waves * HR_BIN_AUTO_PS_WAVE +
+        jb.n * (w.bin.every ? HR_BIN_AUTO_PS_REC_EVERY : HR_BIN_AUTO_PS_REC);
     const unsigned long long binned =
-        HR_BIN_AUTO_PS_BIN + jb.n * HR_BIN_AUTO_PS_BIN_REC + rg.n_words / 5 * HR_BIN_AUTO_PS_BIN_5_WORDS;
-    if (waves > HR_BIN_MAX_WAVES || binned >= per_wave) {  // the same for every thread
+        HR_BIN_AUTO_PS_BIN + jb.n * (w.bin.every ? HR_BIN_AUTO_PS_BIN_REC_EVERY : HR_BIN_AUTO_PS_BIN_REC) + rg.n_words / 5 * HR_BIN_AUTO_PS_BIN_5_WORDS;
+    if (waves > HR_BIN_MAX_WAVES || binned >= per_wave || (w.bin.every && !w.ctl->fresh)) {  // the same for every thread
         if (threadIdx.x == 0) w.ctl->bin_skip = 1u;
         return;
     }
@@ -351,7 +354,9 @@ __device__ void bin_choose(hr_work& w, const hr_jobd& jb, const hr_region_dev& r
     }
     if (fullest) atomicMax(&s_fullest, fullest);
     __syncthreads();
-    if (threadIdx.x == 0 && binned + s_fullest * part * HR_BIN_AUTO_PS_BIN_FULLEST >= per_wave) w.ctl->bin_skip = 1u;
+    if (threadIdx.x == 0 && binned + s_fullest * part *
+                                             (w.bin.every ? HR_BIN_AUTO_PS_BIN_FULLEST_EVERY : HR_BIN_AUTO_PS_BIN_FULLEST) >=
+                                per_wave) w.ctl->bin_skip = 1u;
 }
 static_assert(HR_BIN_AUTO_MAX_N / HR_BIN_SAMPLES < (1ull << 32) && HR_BIN_AUTO_MIN_N >= HR_BIN_SAMPLES, "sample parts");
 static_assert(HR_BIN_SAMPLES <= HR_SMALL_INTERVALS, "the sample's counters fit the interval list");
@@ -444,6 +449,7 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
         w.ctl->n_jobs = 1;
         w.ctl->t0_ns = globaltimer();
         reset_ctl(w.ctl, j0.n_waves);
+        w.ctl->bin_every = w.bin.every;
         if (over) hr_set_error(&rg.error, HR_ERR_CAPACITY);
     }
     if (!over && s_list.n_found <= FOUND) {

@@ -129,3 +129,33 @@ def test_host_trace_wave_limit_counts_over_pieces(hr, monkeypatch):
         with hr.Checker([dict(n_words=WORDS, block_dim=64)]) as ck:
             ck.check_trace_host(0, torch.from_numpy(trace.view(np.uint8)).pin_memory())
             assert hr.STATUS[ck.report(0, cap=0)[1]] == status
+
+
+EVERY = ["taken", "block of 96", "few waves", "hub word", "kernels, clears", "three calls", "a call per kernel",
+         "wide tids", "window", "more segments"]
+
+
+@pytest.mark.parametrize("name", EVERY)
+def test_every_epoch_equals_per_wave(hr, name):
+    """Every-epoch regions: the default against the plain entry point, which is always per-wave."""
+    import torch
+    t, reg, filt, calls = CASES[name]
+    trace = trace_of(len(name) + 100, **t)
+    n_words = WORDS if filt else t.get("words", WORDS)
+    reg = dict(dict(n_words=n_words, block_dim=64, report_mode=hr.REPORT_EVERY_EPOCH), **reg)
+    d = torch.from_numpy(trace.view(np.uint8)).cuda()
+    cuts = [16 * (len(trace) * i // calls) for i in range(calls)] if calls else \
+        [16 * int(i) for i in np.unique(trace["kernel"], return_index=True)[1]]
+    cuts.append(d.numel())
+    told = []
+    for aggregate in (False, True):
+        shadow = torch.full((3 * n_words,), -1, dtype=torch.int64, device="cuda")
+        with hr.Checker([reg], report_capacity=1 << 22, buffers=[shadow]) as ck:
+            if filt:
+                ck.set_filter(0, **filt)
+            for a, b in zip(cuts[:-1], cuts[1:]):
+                ck.check_trace(0, d[a:b], aggregate=aggregate)
+            races, status, n, _ = ck.report(0)
+            told.append((status, n, hr.race_keys(races), ck.counters(0)["accesses"], shadow.cpu().numpy().tobytes()))
+    assert told[0][0] == hr.HR_OK and told[0][1] == len(told[0][2]) > 100
+    assert told[1] == told[0]
