@@ -346,8 +346,13 @@ hr_status hr_destroy(hr_ctx* ctx);
  * tile and whether lanes on the same word are aggregated; even ids aggregate
  * and the odd id after each is the same shape without aggregation.  Until
  * hr_set_variant or hr_autotune chooses one (hr_get_variant then says 0), the
- * library picks the faster checker for each check by its size; races, counts
- * and shadows are the same with every one.  Id 6 is the
+ * library picks the faster checker for each check by its size and, on the
+ * device, its waves and a sample of its records; races, counts and shadows are
+ * the same with every one.  Where that may be the binned one (single traces of 2^18
+ * to 2^27 records on regions of at least 2^20 words), scratch of the size below is
+ * allocated on first use - at most 3 GiB a context and a quarter of the free
+ * memory, and never while `stream` is captured; without it the check takes a
+ * per-wave shape.  Id 6 is the
  * binned checker, which hr_variant_desc reports with zero records per lane and
  * zero consumer warps: the accesses are moved into (4096-word shadow segment,
  * wave) buckets and persistent thread groups apply each segment's buckets to a
@@ -366,9 +371,10 @@ hr_status hr_destroy(hr_ctx* ctx);
  * leaves the region reset.  A variant whose run ends with HR_ERR_CONTENTION or
  * HR_ERR_TIMEOUT (a bound of that variant ran out) is skipped and gets -1 ms;
  * any other error is the trace's, and hr_autotune returns it.
- * Regions in HR_REPORT_EVERY_EPOCH mode always use a checker of their own
- * (variant 3's shape): the variant setting does not apply to them, and
- * hr_autotune on such a region returns HR_ERR_INVALID.
+ * Regions in HR_REPORT_EVERY_EPOCH mode always use checkers of their own (a
+ * per-wave one, and a binned one picked as above when the region's shadow is
+ * new or reset): the variant setting does not apply to them, and hr_autotune on
+ * such a region returns HR_ERR_INVALID.
  */
 uint32_t hr_variant_count(void);
 hr_status hr_variant_desc(uint32_t id, uint32_t* aggregate, uint32_t* records_per_lane, uint32_t* consumer_warps);
