@@ -42,6 +42,8 @@
 //                         is live), its accesses in wave order with a
 //                         shared-memory CAS per access, races appended to the
 //                         region's ring, the segment written back
+// Every-epoch regions whose shadow holds nothing live go the same way, with groups of
+// their own (pe_run).
 // A check with more than HR_BIN_MAX_WAVES waves is not binned: the flag stays
 // clear and the per-wave checker launched after these kernels does the work.
 #include <cooperative_groups.h>
