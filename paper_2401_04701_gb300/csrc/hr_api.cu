@@ -4,6 +4,7 @@
 #include <cstddef>
 #include <cstdlib>
 #include <cstring>
+#include <mutex>
 #include <new>
 #include <vector>
 
@@ -36,6 +37,7 @@ struct RegionHost {
     bool captured = false;                // work was queued inside a stream capture
     bool views = false;                   // a device view was handed out (inline writes possible)
     void* bin_mem = nullptr;              // binned checker tables (allocated by its first check)
+    unsigned long long bin_denied = 0;    // scratch the automatic route could not get (asked for once only)
     hr_bin bin{};                         // carved out of bin_mem; bin.out is its own allocation
 };
 
@@ -88,6 +90,7 @@ struct hr_ctx {
     unsigned test_flags = 0;
     unsigned variant = 0;              // kernel variant of later checks (hr_set_variant / hr_autotune)
     bool chosen = false;               // the caller chose it; else checks may take the binned route
+    std::mutex auto_lock;              // (threads may check different regions at once)
     unsigned long long auto_bytes = 0; // scratch allocated for checks that took that route by themselves
     std::vector<void*> retired;        // buffers outgrown there (checks in flight may still use them)
     cudaStream_t copies = nullptr;     // non-blocking stream for report copies (never waits on user streams)
@@ -331,10 +334,13 @@ static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
     hr_bin_shape(cap_seg, &shape);
     const uint64_t room = (n + n / 8 + 0xFFFFF) & ~0xFFFFFull;  // calls of about one size share a buffer
     const uint64_t bytes = room * sizeof(uint2) + (r.bin_mem ? 0 : hr_bin_table_bytes(cap_seg, HR_BIN_MAX_WAVES + shape.slices - 1));
+    std::lock_guard<std::mutex> lock(ctx->auto_lock);
     size_t free_b = 0, total_b = 0;
+    if (r.bin_denied && bytes >= r.bin_denied) return false;
     if (ctx->auto_bytes + bytes > HR_BIN_AUTO_BYTES || cudaMemGetInfo(&free_b, &total_b) != cudaSuccess ||
         bytes > free_b / 4) {
         (void)cudaGetLastError();
+        r.bin_denied = bytes;
         return false;
     }
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
@@ -344,8 +350,12 @@ static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
     r.bin.out_cap = 0;
     const bool ok = ensure_bin(r, room, s) == HR_OK;
     cudaThreadExchangeStreamCaptureMode(&mode);
-    if (ok) ctx->auto_bytes += bytes;
-    else (void)cudaGetLastError();
+    if (ok) {
+        ctx->auto_bytes += bytes;
+    } else {
+        (void)cudaGetLastError();
+        r.bin_denied = bytes;
+    }
     return ok;
 }
 

@@ -1196,8 +1196,7 @@ namespace {
 template <unsigned CL>
 void shape_of(hr_bin* bin)
 {
-    static unsigned c_cached = 0, s_cached = 0;
-    if (!c_cached) {
+    static const hr_bin shape = [] {  // (threads may ask at once)
         int dev = 0, sms = 0;
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
@@ -1220,17 +1219,20 @@ void shape_of(hr_bin* bin)
             (void)cudaGetLastError();
             clusters = sms / (int)CL;
         }
-        unsigned sub = (unsigned)sms / (unsigned)clusters;
-        if (sub < 1) sub = 1;
-        if (sub > HR_BIN_MAX_SUB) sub = HR_BIN_MAX_SUB;
-        while ((unsigned)clusters * sub > STREAM_THREADS) --sub;
-        s_cached = sub;
-        c_cached = (unsigned)clusters;
-    }
-    bin->cluster = CL;
-    bin->clusters = c_cached;
-    bin->sub = s_cached;
-    bin->slices = c_cached * s_cached;
+        hr_bin b{};
+        b.cluster = CL;
+        b.clusters = (unsigned)clusters;
+        b.sub = (unsigned)sms / (unsigned)clusters;
+        if (b.sub < 1) b.sub = 1;
+        if (b.sub > HR_BIN_MAX_SUB) b.sub = HR_BIN_MAX_SUB;
+        while (b.clusters * b.sub > STREAM_THREADS) --b.sub;
+        b.slices = b.clusters * b.sub;
+        return b;
+    }();
+    bin->cluster = shape.cluster;
+    bin->clusters = shape.clusters;
+    bin->sub = shape.sub;
+    bin->slices = shape.slices;
 }
 
 }  // namespace

@@ -683,19 +683,23 @@ template <bool AGG, int RPL, bool EVERY>
 cudaError_t launch(hr_region_dev* d_regions, const hr_work& w, unsigned long long n, const unsigned char* d_table,
                    cudaStream_t stream)
 {
-    static int sms = 0, per_sm = 0;
-    if (!per_sm) {
+    struct Fit {
+        int sms, per_sm;
+    };
+    static const Fit fit = [] {  // (threads may launch at once)
+        Fit f{0, 0};
         int dev = 0;
         cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, hr_run_kernel<AGG, RPL, EVERY>, CHECK_THREADS, 0);
-        if (per_sm < 1) per_sm = 1;
-    }
+        cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.per_sm, hr_run_kernel<AGG, RPL, EVERY>, CHECK_THREADS, 0);
+        if (f.per_sm < 1) f.per_sm = 1;
+        return f;
+    }();
     // no more warps than the records give items to (one CTA per SM at least, for
     // shadow clears): others would only start, take a ticket and leave
     const unsigned long long items = (n + w.tile - 1) / w.tile, ctas = (items + CONS - 1) / CONS;
-    const unsigned long long full = (unsigned long long)sms * per_sm;
-    const unsigned grid = (unsigned)(ctas > full ? full : ctas < (unsigned)sms ? (unsigned)sms : ctas);
+    const unsigned long long full = (unsigned long long)fit.sms * fit.per_sm;
+    const unsigned grid = (unsigned)(ctas > full ? full : ctas < (unsigned)fit.sms ? (unsigned)fit.sms : ctas);
     hr_run_kernel<AGG, RPL, EVERY><<<grid, CHECK_THREADS, 0, stream>>>(d_regions, w, d_table);
     return cudaGetLastError();
 }
