@@ -33,7 +33,8 @@
  * e.g. T = 16: bc and wc 4 bits each; T = 18: 3 bits each.  The state
  * machine runs on the 8-byte layout; the compact word is only its storage
  * form (hr_expand32 / hr_compress64), so both sizes take the same
- * transitions.  A tid, bc or wc beyond its width is HR_ERR_CLOCK_OVERFLOW.
+ * transitions.  A tid, bc or wc beyond its width is HR_ERR_CLOCK_OVERFLOW; so
+ * is a wc above 255, the 8-byte layout's limit, when W is 9 or 10 (T < 7).
  */
 #ifndef HIRACE_DEVICE_CUH
 #define HIRACE_DEVICE_CUH
@@ -286,8 +287,9 @@ static __device__ __forceinline__ bool hr_monitored(const hr_filter& f, const hr
 /* Whether an access's identity and clocks fit the region's packing. */
 static __device__ __forceinline__ bool hr_fits(uint32_t tid, uint32_t bc, uint32_t wc, const hr_geom& g)
 {
-    if (g.shadow_bytes != 4) return bc <= HR_BC_MAX && wc <= HR_WC_MAX;
-    return (tid >> g.tid_bits) == 0 && (wc >> hr_wc_bits(g)) == 0 && (bc >> hr_bc_bits(g)) == 0;
+    if (bc > HR_BC_MAX || wc > HR_WC_MAX) return false;  /* (a compact form of 4 to 6 tid bits has more than 8 for wc) */
+    return g.shadow_bytes != 4 ||
+           ((tid >> g.tid_bits) == 0 && (wc >> hr_wc_bits(g)) == 0 && (bc >> hr_bc_bits(g)) == 0);
 }
 
 /* compact storage form -> the 8-byte layout */

@@ -965,8 +965,7 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
             // non-absorbing reports: only the EVERY instantiation carries that path
             const bool every = EVERY && g.report_mode == HR_REPORT_EVERY_EPOCH;
             // the wave's clocks fit the region's shadow packing (else every access overflows it)
-            const bool clk_fit = g.shadow_bytes != 4 ? (bc <= HR_BC_MAX && wc <= HR_WC_MAX)
-                                                     : ((wc >> hr_wc_bits(g)) == 0 && (bc >> hr_bc_bits(g)) == 0);
+            const bool clk_fit = hr_fits(0u, bc, wc, g);
             // Phase 1: decode the lane's records, drop or group repeats (warp
             // aggregation), note each access in the warp's slots and issue every
             // shadow load of the tile at once.  When the previous stage is still

@@ -391,8 +391,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
         const hr_record* rec = it.first + (unsigned long long)item * ITEM + lane;
         unsigned n_rec = (unsigned)min((unsigned long long)n_items * ITEM, it.n - (unsigned long long)item * ITEM);
         // the wave's clocks fit the region's shadow packing (else every access overflows it)
-        const bool clk_fit = !sb4 ? (bc <= HR_BC_MAX && wc <= HR_WC_MAX)
-                                  : ((wc >> hr_wc_bits(g)) == 0 && (bc >> hr_bc_bits(g)) == 0);
+        const bool clk_fit = hr_fits(0u, bc, wc, g);
         const bool plain = !it.filtering && !sb4 && clk_fit;  // no filter, every tid and clock fits
         const bool lookup = it.lookup != 0;
         const unsigned bds = g.bd_shift, wss = g.ws_shift;
