@@ -516,7 +516,8 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                     unsigned long long sv = q.o[i];
                     bool done = false;
                     raced = 0;
-                    for (unsigned tries = 0;; ++tries) {
+                    bool spare = (defer >> k) & 1u;  // a deferred access has not tried yet: one CAS beside the cap's
+                    for (unsigned tries = 0;;) {
                         unsigned r = 0;
                         unsigned long long nv;
                         if (AGG && m != (1u << lane)) {
@@ -532,7 +533,8 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                             done = true;
                             break;
                         }
-                        if (tries >= w.cas_cap + ((defer >> k) & 1u)) break;  // (a deferred access has not tried yet)
+                        if (spare) spare = false;
+                        else if (tries++ >= w.cas_cap) break;
                         lc_cas++;
                         const unsigned long long x = hr_shadow_cas(shadow, wd, sv, nv, g);
                         if (x == sv) {

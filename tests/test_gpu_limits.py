@@ -1,4 +1,5 @@
-"""What a check does at its limits: clocks at the edge of the compact packing."""
+"""What a check does at its limits: clocks at the edge of the compact packing and the largest
+retry cap."""
 import numpy as np
 import pytest
 
@@ -42,3 +43,24 @@ def test_compact_warp_clock_limit(hr, tid_bits, how):
                 ck.check_trace(0, to_dev(rec), aggregate=how != "plain")
             _, got, races, _ = ck.report(0)
         assert (hr.STATUS[got], races) == (status, n), wcs
+
+
+@pytest.mark.parametrize("variant", [0, 1, 2, 3])
+@pytest.mark.parametrize("cap", [0xFFFFFFFF, 0xFFFFFFFE, 1 << 20])
+def test_largest_retry_cap(oracle_mod, hr, variant, cap):
+    """A retry cap near the top of its range is no limit: hot words, which every CTA has CASes out
+    for at once, give the oracle's races and no contention."""
+    rng = np.random.default_rng(variant)
+    rec = np.zeros(1 << 16, tg.RECORD)
+    rec["word"] = rng.integers(0, 4, len(rec))
+    rec["tid"] = rng.integers(0, 4096, len(rec))
+    rec["kernel"] = np.arange(len(rec)) * 4 // len(rec)
+    rec["op"] = rng.choice([tg.OP_R, tg.OP_A], len(rec))
+    want = oracle_mod.race_keys(oracle_mod.bruteforce_parallel(rec, 64, 4))
+    with hr.Checker([dict(n_words=4, block_dim=64)]) as ck:
+        ck.set_variant(variant)
+        ck.set_limits(cas_retry_cap=cap)
+        ck.check_trace(0, to_dev(rec))
+        races, status, n, _ = ck.report(0)
+        assert ck.counters(0)["accesses"] == len(rec)
+    assert hr.STATUS[status] == "HR_OK" and n == len(want) and hr.race_keys(races) == want
