@@ -364,6 +364,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
             ok = __shfl_sync(0xffffffffu, ok, 0);
             __syncwarp();
             known = dep;
+            if (!ok) finished -= n_items;  // (not applied, so not done: no later stage may start on it)
             return ok != 0;
         };
         const bool sb4 = g.shadow_bytes == 4;

@@ -1,5 +1,5 @@
-"""What a check does at its limits: clocks at the edge of the compact packing and the largest
-retry cap."""
+"""What a check does at the limits it was given: clocks at the edge of the compact packing, the
+largest retry cap, and a stage wait that runs out."""
 import numpy as np
 import pytest
 
@@ -64,3 +64,28 @@ def test_largest_retry_cap(oracle_mod, hr, variant, cap):
         races, status, n, _ = ck.report(0)
         assert ck.counters(0)["accesses"] == len(rec)
     assert hr.STATUS[status] == "HR_OK" and n == len(want) and hr.race_keys(races) == want
+
+
+@pytest.mark.parametrize("how", ["first", "every"])
+def test_no_access_passes_a_wait_that_ran_out(hr, how):
+    """A stage wait that runs out ends the check there: the items that waited are not counted as
+    done, so no later wave is applied (the hook holds the second stage; the races are in the third)."""
+    lengths = [64, 1, 60_000]
+    rec = np.zeros(sum(lengths), tg.RECORD)
+    rec["bc"] = np.repeat(np.arange(3), lengths)
+    rec["word"] = np.arange(len(rec))
+    rec["tid"] = np.arange(len(rec))
+    rec["op"] = tg.OP_W
+    rec["word"][65:] = np.arange(60_000) // 2    # each word written by two threads of two blocks
+    rec["tid"][65:] = (np.arange(60_000) % 2) * 64
+    for variant in range(4) if how == "first" else [3]:
+        reg = dict(n_words=len(rec), block_dim=64, report_mode=hr.REPORT_EVERY_EPOCH if how == "every" else 0)
+        with hr.Checker([reg]) as ck:
+            ck.set_variant(variant)
+            ck.check_trace(0, to_dev(rec))
+            assert ck.report(0, cap=0)[1:3] == (hr.HR_OK, 30_000)
+            ck.reset(0)
+            ck.set_limits(wait_ns=100_000_000, test_flags=1)
+            ck.check_trace(0, to_dev(rec))
+            _, status, n, _ = ck.report(0, cap=0)
+        assert (hr.STATUS[status], n) == ("HR_ERR_TIMEOUT", 0), variant
