@@ -351,7 +351,7 @@ constexpr unsigned hr_run_tile(unsigned v)
 {
     return 32u * (v == HR_EVERY_EPOCH_VARIANT ? HR_RUN_EVERY_RPL : (unsigned)HR_VARIANTS[v].rpl);
 }
-constexpr unsigned HR_RUN_CLEAR_WORDS = 1u << 13;  // shadow words per clear item
+constexpr unsigned HR_RUN_CLEAR_WORDS = 1u << 13;  // shadow words per clear item, at least
 #ifndef HR_RING_DEPTH
 #define HR_RING_DEPTH 2
 #endif
@@ -367,6 +367,17 @@ constexpr unsigned HR_RUN_CLEAR_WORDS = 1u << 13;  // shadow words per clear ite
 constexpr int HR_RING = HR_RING_DEPTH;                   // tiles in flight in shared memory
 constexpr unsigned HR_TICKET_BATCH = HR_BATCH;           // tiles a producer claims per ticket
 constexpr unsigned HR_CLEAR_WORDS = 1u << 16;  // shadow words per clear item
+// Words of a clear item: `step`, or as many more as leave a clear of n_words words at
+// most HR_CLEAR_ITEMS items.  A check's items are numbered in 32 bits: its clears (one
+// per kernel-tag group, 2^13 at most) then take 2^29 numbers of them; 2^32 words in
+// items of 2^13 would take all 2^32.
+constexpr unsigned HR_CLEAR_ITEMS = 1u << 16;
+__host__ __device__ constexpr unsigned long long hr_clear_words(unsigned long long n_words, unsigned step)
+{
+    const unsigned long long least = (n_words + HR_CLEAR_ITEMS - 1) / HR_CLEAR_ITEMS;
+    return least <= step ? step : (least + step - 1) / step * step;
+}
+static_assert(hr_clear_words(1ull << 32, HR_CLEAR_WORDS) == HR_CLEAR_WORDS, "hr_check_kernel's clear items");
 constexpr unsigned HR_MAX_INTERVALS = 1u << 16;      // pre-pass intervals of a single-trace check
 constexpr unsigned HR_BATCH_INTERVALS = 1u << 18;    // pre-pass intervals of a batch
 constexpr unsigned long long HR_KEY_MASK = 0xFFFFFFFFFFFFull;

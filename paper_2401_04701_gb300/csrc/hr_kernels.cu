@@ -120,7 +120,8 @@ __device__ __forceinline__ void wave_plan(const hr_work& w, const hr_jobd& jb, c
     const unsigned long long end = L + 1 < jb.n_waves ? w.wave_start[g + 1] : jb.n;
     w.wave_end[g] = end;
     *rec_items = (unsigned)((end - w.wave_start[g] + w.tile - 1) / w.tile);
-    *clr_items = *clear ? (unsigned)((rg.n_words + w.clear_words - 1) / w.clear_words) : 0u;
+    const unsigned long long cw = hr_clear_words(rg.n_words, w.clear_words);
+    *clr_items = *clear ? (unsigned)((rg.n_words + cw - 1) / cw) : 0u;
 }
 
 // One job: stages follow its waves; threads take waves in parallel.

@@ -374,9 +374,9 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
             if (!ready && !wait_dep()) break;
             // bytes [bb, be) of the shadow: 16-byte stores, a 4-byte tail
             const unsigned long long sb = g.shadow_bytes;
-            const unsigned long long bb = (unsigned long long)item * HR_RUN_CLEAR_WORDS * sb;
-            const unsigned long long be =
-                min(((unsigned long long)last_word + 1ull) * sb, bb + (unsigned long long)n_items * HR_RUN_CLEAR_WORDS * sb);
+            const unsigned long long n_words = (unsigned long long)last_word + 1ull;
+            const unsigned long long span = hr_clear_words(n_words, HR_RUN_CLEAR_WORDS) * sb;
+            const unsigned long long bb = item * span, be = min(n_words * sb, bb + n_items * span);
             unsigned char* base8 = reinterpret_cast<unsigned char*>(shadow);
             for (unsigned long long i = bb + 16ull * lane; i < be; i += 512ull) {
                 if (i + 16 <= be)
