@@ -53,6 +53,7 @@
 #include <type_traits>
 
 #include "hr_internal.h"
+#include "hr_per_device.h"
 
 namespace cg = cooperative_groups;
 
@@ -1143,14 +1144,17 @@ __global__ void __launch_bounds__(PG_THREADS, 1)
     }
 }
 
-bool g_attrs = false;
-
 }  // namespace
 
 cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const unsigned char* d_table,
                              cudaStream_t stream)
 {
-    if (!g_attrs) {
+    static hr_per_device<int> sm_count;  // (and the kernels' attributes)
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const int sms = sm_count.get(dev, [dev] {
+        int n = 0;
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev);
         // the shared-memory carveout at its maximum (the groups kernel takes nearly all of it)
         for (const void* k : {(const void*)hr_bin_count, (const void*)hr_bin_groups<true>,
                               (const void*)hr_bin_groups<false>, (const void*)hr_bin_groups<false, true>})
@@ -1159,8 +1163,8 @@ cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const u
         cudaFuncSetAttribute(hr_bin_groups<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
         cudaFuncSetAttribute(hr_bin_groups<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
         cudaFuncSetAttribute(hr_bin_groups<false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)PG_SMEM);
-        g_attrs = true;
-    }
+        return n;
+    });
     const hr_bin& b = w.bin;
     if (b.n_seg == 0 || b.n_seg > b.seg_cap || b.n_seg > HR_BIN_MAX_SEGS || b.clusters == 0 || b.sub == 0 ||
         (b.cluster != HR_BIN_CLUSTER_FEW && b.cluster != HR_BIN_CLUSTER) ||
@@ -1177,12 +1181,7 @@ cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const u
     else
         hr_bin_scatter<HR_BIN_CLUSTER><<<b.clusters * HR_BIN_CLUSTER, STREAM_THREADS, sizeof(ScatterSmem<HR_BIN_CLUSTER>),
                                          stream>>>(d_regions, w);
-    static int sms = 0;  // one persistent segment CTA per SM
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
+    // one persistent segment CTA per SM
     if (b.every) hr_bin_groups<false, true><<<sms, PG_THREADS, PG_SMEM, stream>>>(d_regions, w, d_table);
     else if (b.pow2) hr_bin_groups<true><<<sms, PG_THREADS, PG_SMEM, stream>>>(d_regions, w, d_table);
     else hr_bin_groups<false><<<sms, PG_THREADS, PG_SMEM, stream>>>(d_regions, w, d_table);
@@ -1196,9 +1195,11 @@ namespace {
 template <unsigned CL>
 void shape_of(hr_bin* bin)
 {
-    static const hr_bin shape = [] {  // (threads may ask at once)
-        int dev = 0, sms = 0;
-        cudaGetDevice(&dev);
+    static hr_per_device<hr_bin> shapes;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const hr_bin shape = shapes.get(dev, [dev] {
+        int sms = 0;
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms < (int)CL) sms = CL;
         cudaFuncSetAttribute(hr_bin_scatter<CL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1228,7 +1229,7 @@ void shape_of(hr_bin* bin)
         while (b.clusters * b.sub > STREAM_THREADS) --b.sub;
         b.slices = b.clusters * b.sub;
         return b;
-    }();
+    });
     bin->cluster = shape.cluster;
     bin->clusters = shape.clusters;
     bin->sub = shape.sub;

@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "hr_check.cuh"
+#include "hr_per_device.h"
 
 namespace {
 
@@ -1199,14 +1200,13 @@ __global__ void hr_reconfigure_state(hr_region_dev* region, unsigned long long n
 
 __global__ void hr_set_filter_state(hr_region_dev* region, hr_filter filter) { region->filter = filter; }
 
-int g_grid[HR_N_VARIANTS + 1] = {};
+hr_per_device<int> g_grid[HR_N_VARIANTS + 1];
 
 template <bool AGG, int RPL, int CONS, bool EVERY = false>
-int grid_for()
+int grid_for(int dev)
 {
     using S = Shape<RPL, CONS>;
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
+    int sms = 0, per_sm = 0;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(hr_check_kernel<AGG, RPL, CONS, EVERY>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                          (int)S::BYTES);
@@ -1230,18 +1230,19 @@ int hr_check_grid_size(unsigned variant)
 {
     if (variant > HR_EVERY_EPOCH_VARIANT) variant = 0;
     if (variant == HR_BIN_VARIANT) variant = HR_BIN_FALLBACK;
-    int& cached = g_grid[variant];
-    if (cached) return cached;
-    switch (variant) {
-    case 0: cached = grid_for<true, 4, 8>(); break;
-    case 1: cached = grid_for<false, 4, 8>(); break;
-    case 2: cached = grid_for<true, 2, 8>(); break;
-    case 3: cached = grid_for<false, 2, 8>(); break;
-    case 4: cached = grid_for<true, 1, 8>(); break;
-    case 5: cached = grid_for<false, 1, 8>(); break;
-    default: cached = grid_for<false, 2, 8, true>(); break;
-    }
-    return cached;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    return g_grid[variant].get(dev, [&] {
+        switch (variant) {
+        case 0: return grid_for<true, 4, 8>(dev);
+        case 1: return grid_for<false, 4, 8>(dev);
+        case 2: return grid_for<true, 2, 8>(dev);
+        case 3: return grid_for<false, 2, 8>(dev);
+        case 4: return grid_for<true, 1, 8>(dev);
+        case 5: return grid_for<false, 1, 8>(dev);
+        default: return grid_for<false, 2, 8, true>(dev);
+        }
+    });
 }
 
 void hr_plan_intervals(unsigned long long n, unsigned budget, unsigned* G, unsigned* n_int)

@@ -37,6 +37,7 @@
 #include <cuda_runtime.h>
 
 #include "hr_check.cuh"
+#include "hr_per_device.h"
 
 namespace {
 
@@ -688,15 +689,16 @@ cudaError_t launch(hr_region_dev* d_regions, const hr_work& w, unsigned long lon
     struct Fit {
         int sms, per_sm;
     };
-    static const Fit fit = [] {  // (threads may launch at once)
+    static hr_per_device<Fit> fits;
+    int dev = 0;
+    cudaGetDevice(&dev);
+    const Fit fit = fits.get(dev, [dev] {
         Fit f{0, 0};
-        int dev = 0;
-        cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&f.sms, cudaDevAttrMultiProcessorCount, dev);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&f.per_sm, hr_run_kernel<AGG, RPL, EVERY>, CHECK_THREADS, 0);
         if (f.per_sm < 1) f.per_sm = 1;
         return f;
-    }();
+    });
     // no more warps than the records give items to (one CTA per SM at least, for
     // shadow clears): others would only start, take a ticket and leave
     const unsigned long long items = (n + w.tile - 1) / w.tile, ctas = (items + CONS - 1) / CONS;
