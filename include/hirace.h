@@ -179,10 +179,15 @@ hr_status hr_check_trace(hr_ctx* ctx, uint32_t region, const hr_record* d_trace,
 
 /*
  * hr_check_trace_host - hr_check_trace over a trace in HOST memory: the trace
- * is copied in chunks of chunk_records records (0: 2^21, i.e. 32 MB) through
+ * is copied in chunks of chunk_records records through
  * two device staging buffers owned by the context, each chunk's copy (on a
  * copy stream of the context) overlapping the check of the chunk before it on
  * `stream`.  Chunks may cut waves (the shadow stays resident between them).
+ * chunk_records 0 lets the library choose: pieces of 2^21 records (32 MB), or
+ * with the binned variant chosen as many up to 2^24 as make a piece's check
+ * shorter than its copy.  The limit of waves per call then holds for each 2^24
+ * records together; where it is passed, the pieces before are checked and
+ * their races reported beside HR_ERR_CAPACITY.
  * Asynchronous: h_trace must stay valid, and unchanged, until `stream` has
  * passed this call; page-locked memory lets the copies overlap the checks.
  * Growing the staging buffers synchronises the device once.  Not for use

@@ -423,14 +423,17 @@ extern "C" hr_status hr_check_trace_host(hr_ctx* ctx, uint32_t region, const hr_
 {
     if (!valid_region(ctx, region) || (n > 0 && !h_trace) || n >= (1ull << 40)) return HR_ERR_INVALID;
     if (n == 0) return HR_OK;
-    // By default a group of 2^24 records is one unit of the wave limit and travels in
-    // 32 MB pieces: the copy of a piece hides the check of the one before, so only
-    // the last piece's check adds to the copies (18.8M records: 1.43 ms of copies, and
-    // a whole pass of 2.65 ms with one piece per group, 1.88 ms so).  A piece's check
-    // (about 0.1 ms) is shorter than its copy (0.15 ms).
-    const uint64_t group = chunk_records ? chunk_records : 1ull << 24;
-    if (chunk_records == 0) chunk_records = 1ull << 21;
-    if (chunk_records > n) chunk_records = n;
+    // a group of records is one unit of the wave limit and travels in pieces (hr_host_piece)
+    const uint64_t group = chunk_records ? chunk_records : HR_HOST_GROUP;
+    const hr_region_desc& desc = ctx->regions[region].desc;
+    const bool binned = ctx->chosen && ctx->variant == HR_BIN_VARIANT && desc.report_mode == HR_REPORT_FIRST &&
+                        desc.n_words <= (uint64_t)HR_BIN_MAX_SEGS * HR_BIN_SEG;
+    auto piece_at = [&](uint64_t off) {  // records of the pieces of the group that holds record off
+        const uint64_t left = n - off / group * group, len = left < group ? left : group;
+        const uint64_t piece = chunk_records ? chunk_records : hr_host_piece(len, binned, desc.n_words, desc.shadow_bytes);
+        return piece < len ? piece : len;
+    };
+    const uint64_t first = piece_at(0), last = piece_at(n - 1), room = first > last ? first : last;
     cudaStream_t s = (cudaStream_t)stream;
     (void)cudaGetLastError();
     cudaError_t e = cudaSuccess;
@@ -439,22 +442,25 @@ extern "C" hr_status hr_check_trace_host(hr_ctx* ctx, uint32_t region, const hr_
         if (!ctx->copied[b]) e = cudaEventCreateWithFlags(&ctx->copied[b], cudaEventDisableTiming);
         if (e == cudaSuccess && !ctx->used[b]) e = cudaEventCreateWithFlags(&ctx->used[b], cudaEventDisableTiming);
     }
-    if (e == cudaSuccess && chunk_records > ctx->stage_cap) {
+    if (e == cudaSuccess && room > ctx->stage_cap) {
         // earlier calls may still read the old buffers
         e = cudaDeviceSynchronize();
         for (int b = 0; b < 2 && e == cudaSuccess; ++b) {
             cudaFree(ctx->stage_buf[b]);
             ctx->stage_buf[b] = nullptr;
-            e = cudaMalloc(&ctx->stage_buf[b], chunk_records * sizeof(hr_record));
+            e = cudaMalloc(&ctx->stage_buf[b], room * sizeof(hr_record));
         }
-        ctx->stage_cap = e == cudaSuccess ? chunk_records : 0;
+        ctx->stage_cap = e == cudaSuccess ? room : 0;
     }
     if (e != cudaSuccess) return cuda_status(e);
     hr_status st = HR_OK;
-    uint64_t i = 0;
-    for (uint64_t off = 0; off < n && st == HR_OK; off += chunk_records, ++i) {
+    if (binned) st = ensure_bin(ctx->regions[region], room, s);  // (not grown between two pieces)
+    uint64_t i = 0, m = 0;
+    for (uint64_t off = 0; off < n && st == HR_OK; off += m, ++i) {
         const int b = (int)(i & 1);
-        const uint64_t m = n - off < chunk_records ? n - off : chunk_records;
+        const uint64_t piece = piece_at(off), end = off / group * group + group;
+        m = piece < end - off ? piece : end - off;
+        if (m > n - off) m = n - off;
         // the copy into buffer b waits for the check that last read it, the check for the copy
         e = cudaStreamWaitEvent(ctx->h2d, ctx->used[b], 0);
         if (e == cudaSuccess)

@@ -187,6 +187,32 @@ constexpr unsigned long long HR_BIN_AUTO_PS_WAVE = 9000000, HR_BIN_AUTO_PS_REC =
                              HR_BIN_AUTO_PS_BIN_FULLEST = 1600, HR_BIN_AUTO_PS_REC_EVERY = 40,
                              HR_BIN_AUTO_PS_BIN_REC_EVERY = 30, HR_BIN_AUTO_PS_BIN_FULLEST_EVERY = 4000;
 
+// Records of a piece of a trace in host memory, for `n` of them (at most HR_HOST_GROUP,
+// which count together against the wave limit).  The copy of a piece hides the check of
+// the one before, so only the last piece's check adds to the copies, while a piece is
+// checked in less time than it is copied (16 B a record at 211 GB/s: 76 ps).  The
+// per-wave checker touches the words a piece accesses: 2^21 records (0.16 ms of copy)
+// are enough.  So are they where the library picks the checker for each piece.  The
+// chosen binned checker reads and writes the whole shadow with every piece, as only the
+// first one can find it fresh: about 75 us, 18 ps a record and 2.5 ps a word (4.5 ps on
+// the 4-byte shadow).  Its pieces are the smallest equal parts that keep a quarter of the
+// copy's time to spare, in whole MB (copies that start at an odd multiple of 16 B are
+// slower: 6,428 us instead of 6,131 for the first of these traces).  Measured (us a call from page-locked memory; pieces of 2^21,
+// 2^22, 2^23, 2^24): 75.2M records on 2^26 words 10,135, 6,206, 6,124, 6,105 (4-byte
+// shadow 14,721, 8,540, 6,277, 6,357); 37.6M on 2^25 3,707, 3,116, 3,118, 3,251; 9.4M on
+// 2^25 1,190, 1,114, 1,156, 1,071; 18.8M on 2^24 1,668, 1,660, 1,730, 1,808.  By this
+// rule: 6,131 (4-byte 6,277), 3,112, 1,019 and 1,630.
+constexpr unsigned long long HR_HOST_GROUP = 1ull << 24, HR_HOST_PIECE = 1ull << 21;
+constexpr unsigned long long hr_host_piece(unsigned long long n, bool binned, unsigned long long n_words,
+                                           unsigned shadow_bytes)
+{
+    if (!binned) return HR_HOST_PIECE;
+    const unsigned long long check_ps = 75000000ull + n_words * (shadow_bytes == 4 ? 9 : 5) / 2;
+    const unsigned long long least = check_ps * 5 / 4 / (76 - 18);
+    const unsigned long long parts = n / (least > HR_HOST_PIECE ? least : HR_HOST_PIECE);
+    return parts > 1 ? ((n + parts - 1) / parts + 0xFFFFull) & ~0xFFFFull : n;
+}
+
 // Scratch of the binned checker (hr_binned.cu), one per region.  The region's
 // shadow is cut into segments of HR_BIN_SEG words.  The trace is cut into one
 // contiguous slice per streaming CTA, and a slice into parts, one per wave it
