@@ -384,6 +384,7 @@ static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_t
     w.cas_cap = ctx->cas_cap;
     w.test_flags = ctx->test_flags;
     w.views = r.views ? 1u : 0u;
+    w.n_words = r.desc.n_words;
     w.cont = cont ? 1u : 0u;
     w.tell = 1u;
     unsigned variant = ctx->chosen ? ctx->variant : hr_default_variant(n, r.desc.n_words);
@@ -576,6 +577,7 @@ extern "C" hr_status hr_check_batch(hr_ctx* ctx, const hr_job* jobs, uint32_t n_
     if (ctx->profile) pc = take_events(ctx);
     if (ctx->profile) cudaEventRecord(pc.begin, s);
     hr_work w = ctx->batch;
+    w.n_words = ctx->regions[js[0].region].desc.n_words;  // (one job runs as a single trace)
     w.tell = 1u;
     w.wait_ns = ctx->wait_ns;
     w.cas_cap = ctx->cas_cap;

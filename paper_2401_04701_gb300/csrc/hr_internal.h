@@ -267,7 +267,8 @@ struct hr_work {
     unsigned max_intervals;
     unsigned max_jobs;
     unsigned tile;                   // records per work item (set per kernel variant)
-    unsigned clear_words;            // shadow words per clear item (likewise)
+    unsigned long long clear_words;  // shadow words per clear item (likewise)
+    unsigned long long n_words;      // single traces: words of the region
     unsigned consumers;              // per-warp completions per work item
     unsigned cas_cap;                // CAS retries before HR_ERR_CONTENTION
     unsigned long long wait_ns;      // bound of every device-side wait
@@ -396,7 +397,8 @@ constexpr unsigned HR_CLEAR_WORDS = 1u << 16;  // shadow words per clear item
 // Words of a clear item: `step`, or as many more as leave a clear of n_words words at
 // most HR_CLEAR_ITEMS items.  A check's items are numbered in 32 bits: its clears (one
 // per kernel-tag group, 2^13 at most) then take 2^29 numbers of them; 2^32 words in
-// items of 2^13 would take all 2^32.
+// items of 2^13 would take all 2^32.  (Found by the host: the division in hr_run_kernel
+// cost its main loop registers, 3 % of the power-law push.)
 constexpr unsigned HR_CLEAR_ITEMS = 1u << 16;
 __host__ __device__ constexpr unsigned long long hr_clear_words(unsigned long long n_words, unsigned step)
 {

@@ -121,8 +121,7 @@ __device__ __forceinline__ void wave_plan(const hr_work& w, const hr_jobd& jb, c
     const unsigned long long end = L + 1 < jb.n_waves ? w.wave_start[g + 1] : jb.n;
     w.wave_end[g] = end;
     *rec_items = (unsigned)((end - w.wave_start[g] + w.tile - 1) / w.tile);
-    const unsigned long long cw = hr_clear_words(rg.n_words, w.clear_words);
-    *clr_items = *clear ? (unsigned)((rg.n_words + cw - 1) / cw) : 0u;
+    *clr_items = *clear ? (unsigned)((rg.n_words + w.clear_words - 1) / w.clear_words) : 0u;
 }
 
 // One job: stages follow its waves; threads take waves in parallel.
@@ -1272,7 +1271,7 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
     hr_work w = w_in;
     const bool runs = n_jobs == 1 && hr_variant_runs(variant);
     w.tile = runs ? hr_run_tile(variant) : hr_variant_tile(variant);
-    w.clear_words = runs ? HR_RUN_CLEAR_WORDS : HR_CLEAR_WORDS;
+    w.clear_words = runs ? hr_clear_words(w.n_words, HR_RUN_CLEAR_WORDS) : HR_CLEAR_WORDS;
     w.consumers = hr_variant_consumers(variant);
     if (n_jobs == 0 || n_jobs > HR_MAX_BATCH || n_jobs > w.max_jobs) return cudaErrorInvalidValue;
     const unsigned total_int = jobs[n_jobs - 1].int_begin + jobs[n_jobs - 1].n_int;

@@ -111,7 +111,8 @@ extern "C" hr_status hr_check_trace_noalloc(const hr_record* d_trace, uint64_t n
     if (setup_device(dev, &base) != cudaSuccess) return HR_ERR_CUDA;
     cudaStream_t s = (cudaStream_t)stream;
     hr_region_dev* region = (hr_region_dev*)(base + OFF_REGION);
-    const hr_work w = hr_work_at(base + OFF_WORK, 1, HR_MAX_INTERVALS, HR_NOALLOC_MAX_WAVES);
+    hr_work w = hr_work_at(base + OFF_WORK, 1, HR_MAX_INTERVALS, HR_NOALLOC_MAX_WAVES);
+    w.n_words = n_words;
     const hr_geom g = hr_make_geom(block_dim, warp_size);
     hr_noalloc_begin<<<1, 1, 0, s>>>(region, (unsigned long long*)d_shadow, n_words, d_races, race_cap, g);
     cudaError_t e = cudaGetLastError();

@@ -48,6 +48,11 @@ constexpr unsigned SEEN = 2048;                // entries of the CTA's table of 
 constexpr unsigned FLIGHT = 1024;              // entries of the CTA's table of accesses being CASed
 constexpr unsigned MAX_CLAIM = 16;             // items a warp claims at a time, at most
 
+// WarpItem::last of a stage whose wait ran out.  (Taking the items off the warp's count
+// of finished ones instead kept their number in a register: variant 3 spilled, and the
+// power-law push below took 4.86 instead of 4.55 ms.)
+constexpr unsigned LEFT = 2;
+
 // What a warp keeps of its current stage and region, in shared memory: it is
 // the same for all lanes and read once an item, so it costs no registers.
 struct alignas(16) WarpItem {
@@ -270,7 +275,8 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
         __syncwarp();
         if (lane == 0 && finished) {
             hr_stage* st = &w.stages[it.s];
-            if (it.last) {  // the job's last stage: the item that completes it stamps the job's end
+            if (it.last == LEFT) {  // its wait ran out: what was not applied is not done, and no later stage may start
+            } else if (it.last) {   // the job's last stage: the item that completes it stamps the job's end
                 const unsigned prev = atom_add_release(&st->done, finished);
                 if (prev + finished == it.end - it.begin) w.jobs[st->job].done_ns = globaltimer();
             } else {
@@ -362,10 +368,10 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
             if (lane == 0)
                 ok = stage_wait(&w.stages[dep].done, it.dep_need, dep, s_known, &w.ctl->abort,
                                 &regions[it.region].error, w.wait_ns);
+            if (!ok) it.last = LEFT;
             ok = __shfl_sync(0xffffffffu, ok, 0);
             __syncwarp();
             known = dep;
-            if (!ok) finished -= n_items;  // (not applied, so not done: no later stage may start on it)
             return ok != 0;
         };
         const bool sb4 = g.shadow_bytes == 4;
@@ -375,9 +381,9 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
             if (!ready && !wait_dep()) break;
             // bytes [bb, be) of the shadow: 16-byte stores, a 4-byte tail
             const unsigned long long sb = g.shadow_bytes;
-            const unsigned long long n_words = (unsigned long long)last_word + 1ull;
-            const unsigned long long span = hr_clear_words(n_words, HR_RUN_CLEAR_WORDS) * sb;
-            const unsigned long long bb = item * span, be = min(n_words * sb, bb + n_items * span);
+            const unsigned long long span = w.clear_words * sb;
+            const unsigned long long bb = item * span;
+            const unsigned long long be = min(((unsigned long long)last_word + 1ull) * sb, bb + n_items * span);
             unsigned char* base8 = reinterpret_cast<unsigned char*>(shadow);
             for (unsigned long long i = bb + 16ull * lane; i < be; i += 512ull) {
                 if (i + 16 <= be)
@@ -518,8 +524,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                     unsigned long long sv = q.o[i];
                     bool done = false;
                     raced = 0;
-                    bool spare = (defer >> k) & 1u;  // a deferred access has not tried yet: one CAS beside the cap's
-                    for (unsigned tries = 0;;) {
+                    for (unsigned tries = 0;; ++tries) {
                         unsigned r = 0;
                         unsigned long long nv;
                         if (AGG && m != (1u << lane)) {
@@ -535,8 +540,8 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
                             done = true;
                             break;
                         }
-                        if (spare) spare = false;
-                        else if (tries++ >= w.cas_cap) break;
+                        // (a deferred access has not tried yet: one CAS beside the cap's)
+                        if (tries > w.cas_cap || (tries == w.cas_cap && !((defer >> k) & 1u))) break;
                         lc_cas++;
                         const unsigned long long x = hr_shadow_cas(shadow, wd, sv, nv, g);
                         if (x == sv) {
