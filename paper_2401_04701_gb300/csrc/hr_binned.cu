@@ -53,6 +53,7 @@
 #include <type_traits>
 
 #include "hr_internal.h"
+#include "hr_launch.cuh"
 #include "hr_per_device.h"
 
 namespace cg = cooperative_groups;
@@ -270,6 +271,7 @@ __global__ void __launch_bounds__(STREAM_THREADS) hr_bin_count(hr_region_dev* __
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     StreamSmem& S = *reinterpret_cast<StreamSmem*>(smem_raw);
+    hr_grid_wait();
     if (!bin_fits(w.ctl)) return;
     const unsigned W = w.ctl->n_waves;
     const hr_jobd jb = w.jobs[0];
@@ -332,6 +334,7 @@ __global__ void __launch_bounds__(STREAM_THREADS) hr_bin_count(hr_region_dev* __
 __global__ void __launch_bounds__(SCAN_THREADS) hr_bin_scan_sums(hr_work w)
 {
     __shared__ unsigned s_warp[32];
+    hr_grid_wait();
     if (!bin_fits(w.ctl)) return;
     if (blockIdx.x == 0) {
         // a wave's shadow clear is the stage right before its record stage
@@ -400,6 +403,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) hr_bin_scan_sums(hr_work w)
 __global__ void __launch_bounds__(SCAN_THREADS) hr_bin_scan(hr_work w)
 {
     __shared__ unsigned s_warp[32];
+    hr_grid_wait();
     if (!hr_bin_taken(w.ctl)) return;
     const unsigned long long E = (unsigned long long)w.bin.n_seg * w.ctl->bin_parts;
     const unsigned long long b0 = (unsigned long long)blockIdx.x * HR_BIN_SCAN;
@@ -466,6 +470,7 @@ __global__ void __cluster_dims__(CL, 1, 1) __launch_bounds__(STREAM_THREADS)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     auto& S = *reinterpret_cast<ScatterSmem<CL>*>(smem_raw);
     cg::cluster_group cluster = cg::this_cluster();
+    hr_grid_wait();
     if (!hr_bin_taken(w.ctl)) return;  // the same for every CTA: no remote access happens
     const unsigned W = w.ctl->n_waves, P = w.ctl->bin_parts;
     const hr_jobd jb = w.jobs[0];
@@ -1090,6 +1095,7 @@ __global__ void __launch_bounds__(PG_THREADS, 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     PCommon& C = *reinterpret_cast<PCommon*>(smem_raw);
     unsigned char* gbase = smem_raw + sizeof(PCommon);
+    hr_grid_wait();
     if (!hr_bin_taken(w.ctl)) return;
     const hr_jobd jb = w.jobs[0];
     hr_region_dev* rg = regions + jb.region;
@@ -1172,19 +1178,18 @@ cudaError_t hr_launch_binned(hr_region_dev* d_regions, const hr_work& w, const u
         b.part_cap < HR_BIN_MAX_WAVES + b.slices - 1)
         return cudaErrorInvalidValue;
     const unsigned scan_blocks = (unsigned)(((unsigned long long)b.n_seg * b.part_cap + HR_BIN_SCAN - 1) / HR_BIN_SCAN);
-    hr_bin_count<<<b.slices, STREAM_THREADS, STREAM_SMEM, stream>>>(d_regions, w);
-    hr_bin_scan_sums<<<scan_blocks, SCAN_THREADS, 0, stream>>>(w);
-    hr_bin_scan<<<scan_blocks, SCAN_THREADS, 0, stream>>>(w);
+    hr_launch(hr_bin_count, b.slices, STREAM_THREADS, STREAM_SMEM, stream, d_regions, w);
+    hr_launch(hr_bin_scan_sums, scan_blocks, SCAN_THREADS, 0, stream, w);
+    hr_launch(hr_bin_scan, scan_blocks, SCAN_THREADS, 0, stream, w);
     if (b.cluster == HR_BIN_CLUSTER_FEW)
-        hr_bin_scatter<HR_BIN_CLUSTER_FEW><<<b.clusters * HR_BIN_CLUSTER_FEW, STREAM_THREADS,
-                                             sizeof(ScatterSmem<HR_BIN_CLUSTER_FEW>), stream>>>(d_regions, w);
+        hr_launch(hr_bin_scatter<HR_BIN_CLUSTER_FEW>, b.clusters * HR_BIN_CLUSTER_FEW, STREAM_THREADS,
+                  sizeof(ScatterSmem<HR_BIN_CLUSTER_FEW>), stream, d_regions, w);
     else
-        hr_bin_scatter<HR_BIN_CLUSTER><<<b.clusters * HR_BIN_CLUSTER, STREAM_THREADS, sizeof(ScatterSmem<HR_BIN_CLUSTER>),
-                                         stream>>>(d_regions, w);
+        hr_launch(hr_bin_scatter<HR_BIN_CLUSTER>, b.clusters * HR_BIN_CLUSTER, STREAM_THREADS,
+                  sizeof(ScatterSmem<HR_BIN_CLUSTER>), stream, d_regions, w);
     // one persistent segment CTA per SM
-    if (b.every) hr_bin_groups<false, true><<<sms, PG_THREADS, PG_SMEM, stream>>>(d_regions, w, d_table);
-    else if (b.pow2) hr_bin_groups<true><<<sms, PG_THREADS, PG_SMEM, stream>>>(d_regions, w, d_table);
-    else hr_bin_groups<false><<<sms, PG_THREADS, PG_SMEM, stream>>>(d_regions, w, d_table);
+    const auto groups = b.every ? hr_bin_groups<false, true> : b.pow2 ? hr_bin_groups<true> : hr_bin_groups<false>;
+    hr_launch(groups, (unsigned)sms, PG_THREADS, PG_SMEM, stream, d_regions, w, d_table);
     return cudaGetLastError();
 }
 

@@ -161,18 +161,20 @@ __host__ __device__ inline bool hr_bin_taken(const hr_ctl* c)
 
 // The automatic route: a check for which no variant was chosen takes the binned
 // checker when its pre-pass expects that to be faster, and the count pass meets no
-// error.  The expectation, in picoseconds: the per-wave checker
-// needs about 9 us a wave and 28 ps a record; the binned one 75 us, 18 ps a record,
-// 2.4 ps a word of the region (its shadow is written, and read unless nothing in it
-// is live) and 1.6 ns an access of the fullest segment (one thread group applies
-// it), which a sample of the records estimates.  Measured on global-memory traces
-// (us a call, pre-pass included, per-wave variant 0 / binned): 32 waves, 0.29M
-// records on 2^20 words 289 / 100, 1.18M 296 / 112, 4.7M on 2^22 words 362 / 151,
-// 75.2M on 2^26 words 2145 / 1304; 8 waves, 1.18M on 2^22 words 113 / 103; 4 waves,
-// 0.59M on 2^22 words 70 / 87, 2.35M on 2^24 words 109 / 152; 1 wave, 2.35M on
-// 2^26 words 95 / 267.  A check that the pre-pass leaves to the per-wave checker
-// pays about 20 us for the binned kernels that find nothing to do; that counts on the
-// per-wave checker's side, and smaller checks and regions never get there.
+// error.  The expectation, in picoseconds: the per-wave checker needs 20 us, 9 us a
+// wave and 28 ps a record; the binned one 75 us, 18 ps a record, 2.4 ps a word of the
+// region (its shadow is written, and read unless nothing in it is live) and 1.6 ns an
+// access of the fullest segment (one thread group applies it), which a sample of the
+// records estimates.  The per-wave figures are those of variant 0 with ordinary
+// launches; the shapes that run now take about 6 us a wave, so near break-even the
+// binned checker is taken a little early.  Measured on global-memory traces (us a call,
+// pre-pass included, per-wave variants 1 and 3 / binned / what the rule gives): 32 waves,
+// 0.29M records on 2^20 words 234 and 201 / 102 / 94, 4.7M on 2^22 words 330 and 407 /
+// 148 / 143, 75.2M on 2^26 words 1,967 and 2,135 / 1,315 / 1,291; 8 waves, 0.26M on
+// 2^22 words 92 and 82 / 80 / 71; 4 waves, 0.57M on 2^22 words 66 and 72 / 79 / 75; one
+// wave, 0.26M on 2^22 words 34 and 38 / 72 / 43.  A check that the pre-pass leaves to the
+// per-wave checker pays about 6 us for the binned kernels that find nothing to do;
+// smaller checks and regions never get there.
 // Every-epoch regions take it when nothing in their shadow is live: there the
 // per-wave checker needs 40 ps a record and the binned one 30 ps (pre-pass and check,
 // 32 waves: 4.7M records 565 and 245 us, 18.8M 1043 and about 620 us).

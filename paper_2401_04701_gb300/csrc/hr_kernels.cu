@@ -22,6 +22,7 @@
 #include <cuda_runtime.h>
 
 #include "hr_check.cuh"
+#include "hr_launch.cuh"
 #include "hr_per_device.h"
 
 namespace {
@@ -828,6 +829,7 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
     hr_filter* s_filt = reinterpret_cast<hr_filter*>(s_geom + HR_CONSUMERS);        // [HR_CONSUMERS]
 
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    // the table and the ring's barriers, while the kernel before this one ends
     for (unsigned i = threadIdx.x; i < 256; i += HR_THREADS)
         reinterpret_cast<uint2*>(s_table)[i] = reinterpret_cast<const uint2*>(gtable)[i];
     if (threadIdx.x == 0) {
@@ -838,6 +840,7 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
         for (int b = 0; b < 2 * HR_RING; ++b) s_fin[b] = 0;
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
+    hr_grid_wait();
     __syncthreads();
 
     if (wid == HR_CONSUMERS) {
@@ -1144,11 +1147,12 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
     flush();
 }
 
-// The jobs' reports to the host's copies, after a check.  A launch of its own (about
+// The jobs' reports to the host's copies, after a check.  A launch of its own (1 to
 // 3 us): at the end of the checkers it cost their main loops registers (power-law
 // push of 2^22 vertices 4.54 -> 4.85 ms, tree reduction of 1M records 77 -> 88 us).
 __global__ void hr_tell(const hr_region_dev* regions, const hr_jobd* jobs, const hr_ctl* ctl)
 {
+    hr_grid_wait();
     for (unsigned j = threadIdx.x; j < ctl->n_jobs; j += blockDim.x) {
         const hr_region_dev& rg = regions[jobs[j].region];
         hr_told t;
@@ -1220,7 +1224,7 @@ void launch_variant(int grid, hr_region_dev* d_regions, const hr_work& w, const 
                     cudaStream_t stream)
 {
     using S = Shape<RPL, CONS>;
-    hr_check_kernel<AGG, RPL, CONS, EVERY><<<grid, S::THREADS, S::BYTES, stream>>>(d_regions, w, d_table);
+    hr_launch(hr_check_kernel<AGG, RPL, CONS, EVERY>, (unsigned)grid, S::THREADS, S::BYTES, stream, d_regions, w, d_table);
 }
 
 }  // namespace
@@ -1255,7 +1259,7 @@ void hr_plan_intervals(unsigned long long n, unsigned budget, unsigned* G, unsig
 
 static cudaError_t launch_tell(hr_region_dev* d_regions, const hr_work& w, unsigned n_jobs, cudaStream_t stream)
 {
-    if (w.tell) hr_tell<<<1, n_jobs < 32 ? 32 : 256, 0, stream>>>(d_regions, w.jobs, w.ctl);
+    if (w.tell) hr_launch(hr_tell, 1, n_jobs < 32 ? 32 : 256, 0, stream, d_regions, w.jobs, w.ctl);
     return cudaGetLastError();
 }
 

@@ -37,6 +37,7 @@
 #include <cuda_runtime.h>
 
 #include "hr_check.cuh"
+#include "hr_launch.cuh"
 #include "hr_per_device.h"
 
 namespace {
@@ -232,14 +233,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
     __shared__ unsigned s_first;
 
     const unsigned lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->total_items;  // binned: the work is done already
-    if (total == 0) return;
-    // items per claim: enough to keep the ticket counter out of the way, few
-    // enough that a stage's items spread over all warps
-    const unsigned claim =
-        (unsigned)max(1ull, min((unsigned long long)MAX_CLAIM,
-                                total / ((unsigned long long)w.ctl->n_stages * gridDim.x * (CONS * 2u))));
-    if (threadIdx.x == 0) s_first = atomicAdd(&w.ctl->ticket, CONS * claim);
+    // the tables, while the kernel before this one ends
     for (unsigned i = threadIdx.x; i < 128; i += CHECK_THREADS)
         reinterpret_cast<uint4*>(s_table)[i] = reinterpret_cast<const uint4*>(gtable)[i];
     for (unsigned i = threadIdx.x; i < KNOWN; i += CHECK_THREADS) s_known[i] = 0u;
@@ -248,6 +242,15 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
         for (unsigned i = threadIdx.x; i < 2048; i += CHECK_THREADS) s_abs[i] = (unsigned char)absorbs(gtable, i);
         for (unsigned i = threadIdx.x; i < FLIGHT; i += CHECK_THREADS) s_flight[i] = 0u;
     }
+    hr_grid_wait();
+    const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->total_items;  // binned: the work is done already
+    if (total == 0) return;
+    // items per claim: enough to keep the ticket counter out of the way, few
+    // enough that a stage's items spread over all warps
+    const unsigned claim =
+        (unsigned)max(1ull, min((unsigned long long)MAX_CLAIM,
+                                total / ((unsigned long long)w.ctl->n_stages * gridDim.x * (CONS * 2u))));
+    if (threadIdx.x == 0) s_first = atomicAdd(&w.ctl->ticket, CONS * claim);
     WarpItem& it = s_item[wid];
     if (lane == 0) {
         it.region = ~0u;  // (nothing is counted before the first region is set)
@@ -709,8 +712,7 @@ cudaError_t launch(hr_region_dev* d_regions, const hr_work& w, unsigned long lon
     const unsigned long long items = (n + w.tile - 1) / w.tile, ctas = (items + CONS - 1) / CONS;
     const unsigned long long full = (unsigned long long)fit.sms * fit.per_sm;
     const unsigned grid = (unsigned)(ctas > full ? full : ctas < (unsigned)fit.sms ? (unsigned)fit.sms : ctas);
-    hr_run_kernel<AGG, RPL, EVERY><<<grid, CHECK_THREADS, 0, stream>>>(d_regions, w, d_table);
-    return cudaGetLastError();
+    return hr_launch(hr_run_kernel<AGG, RPL, EVERY>, grid, CHECK_THREADS, 0, stream, d_regions, w, d_table);
 }
 
 }  // namespace
