@@ -423,7 +423,8 @@ hr_status hr_profile_read(hr_ctx* ctx, double* check_ms, double* prepass_ms, uin
  * on an implicit device synchronisation.  No context is needed and nothing is
  * allocated: no cudaMalloc, cudaFree or allocating library routine is called.
  *   d_trace   n records, device memory, same rules as hr_check_trace
- *   d_shadow  n_words 8-byte shadow values, caller-owned device memory.  Each
+ *   d_shadow  n_words 8-byte shadow values, caller-owned device memory at a
+ *             multiple of 8 bytes (16 clears it with wider stores).  Each
  *             call checks one complete trace as a fresh region: before the
  *             trace's first wave the call clears d_shadow (every word INIT),
  *             so what an earlier call or the caller left there does not

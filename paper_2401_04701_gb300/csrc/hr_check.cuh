@@ -31,6 +31,25 @@ __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v)
     asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
+// Bytes [bb, be) of a shadow to zero (one warp; bb a multiple of 16): 16-byte stores and a
+// 4-byte tail.  hr_check_trace_noalloc takes a shadow at any multiple of 8: 8-byte stores
+// then (its values are 8 bytes).
+__device__ __forceinline__ void clear_bytes(void* shadow, unsigned long long bb, unsigned long long be, unsigned lane)
+{
+    unsigned char* const p = static_cast<unsigned char*>(shadow);
+    if (reinterpret_cast<unsigned long long>(p) & 15ull) {
+        for (unsigned long long i = bb + 8ull * lane; i < be; i += 256ull)
+            *reinterpret_cast<unsigned long long*>(p + i) = 0ull;
+        return;
+    }
+    for (unsigned long long i = bb + 16ull * lane; i < be; i += 512ull) {
+        if (i + 16 <= be)
+            *reinterpret_cast<ulonglong2*>(p + i) = make_ulonglong2(0ull, 0ull);
+        else
+            for (unsigned long long j = i; j < be; j += 4) *reinterpret_cast<unsigned*>(p + j) = 0u;
+    }
+}
+
 // Every-epoch mode for a lane's RPL accesses at once (bit k of `act`: slot k
 // holds one): the steps of hr_ep_apply, each over every slot before the next,
 // so each step costs one round trip for all of them and one fence serves them

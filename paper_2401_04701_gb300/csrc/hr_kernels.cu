@@ -950,18 +950,11 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
 
         if (t_type == HR_STAGE_CLEAR && !t_skip) {
             if (!ready && !wait_dep(t_dep, t_need)) break;
-            // bytes [bb, be) of the shadow: 16-byte stores, a 4-byte tail
             const unsigned long long sb = g.shadow_bytes;
             const unsigned long long span = (unsigned long long)(HR_CLEAR_WORDS / HR_CONSUMERS) * sb;
             const unsigned long long bb = (unsigned long long)t_item * HR_CLEAR_WORDS * sb + wid * span;
             const unsigned long long be = min(n_words * sb, bb + span);
-            unsigned char* base8 = reinterpret_cast<unsigned char*>(shadow);
-            for (unsigned long long i = bb + 16ull * lane; i < be; i += 512ull) {
-                if (i + 16 <= be)
-                    *reinterpret_cast<ulonglong2*>(base8 + i) = make_ulonglong2(0ull, 0ull);
-                else
-                    for (unsigned long long j = i; j < be; j += 4) *reinterpret_cast<unsigned*>(base8 + j) = 0u;
-            }
+            clear_bytes(shadow, bb, be, lane);
         } else if (records) {
             const unsigned bc = bcwc >> 16;
             const unsigned wc = bcwc & 0xFFFFu;

@@ -101,7 +101,7 @@ extern "C" hr_status hr_check_trace_noalloc(const hr_record* d_trace, uint64_t n
                                             hr_stream_t stream)
 {
     if ((n > 0 && !d_trace) || !d_shadow || !d_result || (race_cap > 0 && !d_races)) return HR_ERR_INVALID;
-    if (((uintptr_t)d_trace & 15u) != 0) return HR_ERR_INVALID;
+    if (((uintptr_t)d_trace & 15u) != 0 || ((uintptr_t)d_shadow & 7u) != 0) return HR_ERR_INVALID;
     if (n_words == 0 || n_words > (1ull << 32) || block_dim == 0 || warp_size == 0 || warp_size > 32 ||
         n >= (1ull << 40))
         return HR_ERR_INVALID;

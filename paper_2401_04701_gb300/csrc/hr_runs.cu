@@ -382,18 +382,11 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
         const unsigned last_word = it.last_word;
         if (it.type == HR_STAGE_CLEAR) {
             if (!ready && !wait_dep()) break;
-            // bytes [bb, be) of the shadow: 16-byte stores, a 4-byte tail
             const unsigned long long sb = g.shadow_bytes;
             const unsigned long long span = w.clear_words * sb;
             const unsigned long long bb = item * span;
             const unsigned long long be = min(((unsigned long long)last_word + 1ull) * sb, bb + n_items * span);
-            unsigned char* base8 = reinterpret_cast<unsigned char*>(shadow);
-            for (unsigned long long i = bb + 16ull * lane; i < be; i += 512ull) {
-                if (i + 16 <= be)
-                    *reinterpret_cast<ulonglong2*>(base8 + i) = make_ulonglong2(0ull, 0ull);
-                else
-                    for (unsigned long long j = i; j < be; j += 4) *reinterpret_cast<unsigned*>(base8 + j) = 0u;
-            }
+            clear_bytes(shadow, bb, be, lane);
             continue;
         }
         const unsigned kern = (unsigned)(it.key >> 32), bcwc = (unsigned)it.key;

@@ -1,5 +1,5 @@
-"""What a check does at the limits it was given: clocks at the edge of the compact packing, the
-largest retry cap, and a stage wait that runs out."""
+"""What a check does at its limits: clocks at the edge of the compact packing, the largest retry
+cap, a stage wait that runs out, and the alignment of a shadow handed in."""
 import numpy as np
 import pytest
 
@@ -89,3 +89,37 @@ def test_no_access_passes_a_wait_that_ran_out(hr, how):
             ck.check_trace(0, to_dev(rec))
             _, status, n, _ = ck.report(0, cap=0)
         assert (hr.STATUS[status], n) == ("HR_ERR_TIMEOUT", 0), variant
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 3])
+@pytest.mark.parametrize("words", [1, 2, 8191, 16384, 40_001])
+def test_noalloc_shadow_at_any_multiple_of_8(oracle_mod, hr, words, offset):
+    """The allocation-free check clears exactly its n_words values wherever an 8-byte shadow lies,
+    and refuses one that no 64-bit atomic could work on."""
+    import ctypes
+    import torch
+    rng = np.random.default_rng(words)
+    rec = np.zeros(5000, tg.RECORD)
+    rec["word"], rec["tid"] = rng.integers(0, words, len(rec)), rng.integers(0, 512, len(rec))
+    rec["op"] = rng.integers(0, 2, len(rec))
+    rec["kernel"] = np.arange(len(rec)) * 20 // len(rec)      # (clears between the tag groups, too)
+    want = oracle_mod.race_keys(oracle_mod.bruteforce_parallel(rec, 64, words))
+    d, buf = to_dev(rec), torch.full((words + 8,), -7, dtype=torch.int64, device="cuda")
+    races = torch.zeros(1 << 20, dtype=torch.uint8, device="cuda")
+    result = torch.zeros(2, dtype=torch.int64, device="cuda")
+    fn = hr.load_library().hr_check_trace_noalloc
+    P, u32, u64 = ctypes.c_void_p, ctypes.c_uint32, ctypes.c_uint64
+    fn.argtypes, fn.restype = [P, u64, P, u64, u32, u32, P, u64, P, P], ctypes.c_int
+
+    def call(shadow):
+        return fn(d.data_ptr(), len(rec), shadow, words, 64, 32, races.data_ptr(), 1 << 16, result.data_ptr(),
+                  torch.cuda.current_stream().cuda_stream)
+
+    assert call(buf.data_ptr() + 8 * offset + 4) == 1           # HR_ERR_INVALID, before any launch
+    assert call(buf.data_ptr() + 8 * offset) == 0
+    torch.cuda.synchronize()
+    n = int(result[0])
+    assert int(result[1]) == 0 and n == len(want)
+    assert hr.race_keys(races.cpu().numpy().view(hr.RACE_DTYPE)[:n]) == want
+    assert (buf[:offset] == -7).all() and (buf[offset + words:] == -7).all()
+    assert (buf[offset:offset + words] != -7).all()
