@@ -36,6 +36,8 @@ struct RegionHost {
     cudaEvent_t done = nullptr;           // recorded after every call on the region
     bool captured = false;                // work was queued inside a stream capture
     bool views = false;                   // a device view was handed out (inline writes possible)
+    bool fresh = true;                    // nothing was queued since init or a reset (a graph's replay is
+                                          // not seen: a hint, the pre-pass knows)
     void* bin_mem = nullptr;              // binned checker tables (allocated by its first check)
     unsigned long long bin_denied = 0;    // scratch the automatic route could not get (asked for once only)
     hr_bin bin{};                         // carved out of bin_mem; bin.out is its own allocation
@@ -325,7 +327,8 @@ static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
     const uint64_t n_seg = (r.desc.n_words + HR_BIN_SEG - 1) / HR_BIN_SEG;
     const bool every = r.desc.report_mode == HR_REPORT_EVERY_EPOCH;  // (the variant does not apply to them)
     if ((ctx->chosen && !every) || n < HR_BIN_AUTO_MIN_N || n > HR_BIN_AUTO_MAX_N ||
-        n_seg < HR_BIN_AUTO_SEGS || cap_seg > HR_BIN_MAX_SEGS || ctx->test_flags || ctx->cas_cap < HR_DEFAULT_CAS_CAP)
+        n_seg < HR_BIN_AUTO_SEGS || cap_seg > HR_BIN_MAX_SEGS || ctx->test_flags || ctx->cas_cap < HR_DEFAULT_CAS_CAP ||
+        (every && !r.fresh))  // (every-epoch regions take it on an empty shadow only)
         return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
@@ -409,6 +412,7 @@ static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_t
         pc.launches = launches;
         ctx->calls.push_back(pc);
     }
+    r.fresh = false;
     if (e == cudaSuccess) e = mark_done(r, s);
     return cuda_status(e);
 }
@@ -593,8 +597,10 @@ extern "C" hr_status hr_check_batch(hr_ctx* ctx, const hr_job* jobs, uint32_t n_
         pc.launches = launches;
         ctx->calls.push_back(pc);
     }
-    for (auto& d : js)
+    for (auto& d : js) {
+        ctx->regions[d.region].fresh = false;
         if (e == cudaSuccess) e = mark_done(ctx->regions[d.region], s);
+    }
     return cuda_status(e);
 }
 
@@ -612,6 +618,7 @@ extern "C" hr_status hr_sync(hr_ctx* ctx, uint32_t region, uint32_t scope, hr_st
     if (e == cudaSuccess) e = hr_launch_sync_kernel(r.d, s);
     if (e == cudaSuccess) e = mark_done(r, s);
     if (e == cudaSuccess) r.kernel++;
+    r.fresh = false;
     return cuda_status(e);
 }
 
@@ -670,6 +677,7 @@ extern "C" hr_status hr_reset(hr_ctx* ctx, uint32_t region, hr_stream_t stream)
     cudaError_t e = hr_launch_reset(r.d, r.shadow, r.desc.n_words * hr_desc_shadow_bytes(r.desc), s);
     if (e == cudaSuccess) e = mark_done(r, s);
     r.kernel = 0;
+    r.fresh = true;
     return cuda_status(e);
 }
 
@@ -691,6 +699,7 @@ extern "C" hr_status hr_region_reconfigure(hr_ctx* ctx, uint32_t region, uint64_
     if (e == cudaSuccess) e = hr_launch_reset(r.d, r.shadow, n_words * hr_desc_shadow_bytes(r.desc), s);
     if (e == cudaSuccess) e = mark_done(r, s);
     r.kernel = 0;
+    r.fresh = true;
     return cuda_status(e);
 }
 

@@ -145,6 +145,7 @@ struct hr_ctl {
     unsigned bin_count;    // binned checker: accesses counted into buckets
     unsigned bin_skip;     // automatic route: 1: the pre-pass left this check to the per-wave checker
     unsigned bin_every;    // 1: every-epoch region (binned only in the 4-byte working form)
+    unsigned run_items;    // total_items where hr_run_kernel has them, 0 where hr_check_kernel does
     unsigned bin_err;      // automatic route: 1: the count pass met an error (the per-wave checker then
                            // does the check, and reports it)
 };
@@ -269,6 +270,7 @@ struct hr_work {
     unsigned max_intervals;
     unsigned max_jobs;
     unsigned tile;                   // records per work item (set per kernel variant)
+    unsigned check_tile;             // 0, or both per-wave checkers are launched: hr_check_kernel's records per item
     unsigned long long clear_words;  // shadow words per clear item (likewise)
     unsigned long long n_words;      // single traces: words of the region
     unsigned consumers;              // per-warp completions per work item
@@ -371,11 +373,30 @@ constexpr unsigned hr_variant_tile(unsigned v)
            : v == HR_BIN_VARIANT       ? hr_variant_tile(HR_BIN_FALLBACK)
                                        : HR_VARIANTS[v].consumers * 32u * HR_VARIANTS[v].rpl;
 }
-// hr_runs.cu: which checks of one trace it takes, and its work items (one step of
-// a warp).  The others run hr_check_kernel: batches, and the shapes of variants 4
-// and 5 (hr_runs.cu says what each is better at).
+// The checker of a single trace: hr_run_kernel (hr_runs.cu) for variants 0 to 3 and
+// every-epoch regions, hr_check_kernel for variants 4 and 5, or the one that the trace's
+// waves are better for.  The host does not know the waves, so both are launched then and
+// the pre-pass leaves one of them no items (about 1 us).
+//
+// Every-epoch regions (us, hr_check_kernel with 2 records a lane / hr_run_kernel with 4;
+// waves of n records): 0.29M records in 32 waves 335 / 457, 1.03M in 32 307 / 390, 2.35M
+// in 32 447 / 512; 3.5M in 32 587 / 539, 18.8M in 32 1,446 / 1,055, 37.6M in 32 2,072 /
+// 1,900; 9.2M in 4 512 / 633, 75.2M in 32 3,650 / 3,928; 0.57M in 4 87 / 104, 2.3M in 4
+// 211 / 192.
 constexpr unsigned HR_RUN_EVERY_RPL = 4;  // records per lane in every-epoch regions
-constexpr bool hr_variant_runs(unsigned v) { return v < 4 || v == HR_EVERY_EPOCH_VARIANT; }
+enum hr_route { HR_ROUTE_RUNS, HR_ROUTE_TILES, HR_ROUTE_BY_WAVES };
+constexpr unsigned long long HR_EVERY_RUNS_MIN_N = 1ull << 21;  // records, and of a wave:
+constexpr unsigned long long HR_EVERY_RUNS_MIN_WAVE = 98304, HR_EVERY_RUNS_MAX_WAVE = 1250000;
+constexpr hr_route hr_single_route(unsigned v, unsigned long long n)
+{
+    if (v == HR_EVERY_EPOCH_VARIANT) return n < HR_EVERY_RUNS_MIN_N ? HR_ROUTE_TILES : HR_ROUTE_BY_WAVES;
+    return v < 4 ? HR_ROUTE_RUNS : HR_ROUTE_TILES;
+}
+// HR_ROUTE_BY_WAVES: whether hr_check_kernel takes a trace of n records in `waves` waves
+__host__ __device__ constexpr bool hr_waves_tiled(unsigned long long n, unsigned waves)
+{
+    return n < waves * HR_EVERY_RUNS_MIN_WAVE || n > waves * HR_EVERY_RUNS_MAX_WAVE;
+}
 constexpr unsigned hr_run_tile(unsigned v)
 {
     return 32u * (v == HR_EVERY_EPOCH_VARIANT ? HR_RUN_EVERY_RPL : (unsigned)HR_VARIANTS[v].rpl);
@@ -415,12 +436,13 @@ constexpr unsigned long long HR_KEY_MASK = 0xFFFFFFFFFFFFull;
 // kernel launch helpers (hr_kernels.cu)
 // Check n_jobs jobs (1..HR_MAX_BATCH) on the regions of d_regions with the
 // scratch w.  Jobs must name distinct regions and hold n > 0 records.
-// *launches (if not NULL) receives the kernels launched: 3 for a single trace
-// (8 with the binned checker), 5 for a batch; one fewer without w.tell.
+// *launches (if not NULL) receives the kernels launched: 3 for a single trace (one more
+// with both per-wave checkers, five with the binned one), 5 for a batch; one fewer
+// without w.tell.
 cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w, const hr_jobd* jobs, unsigned n_jobs,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream,
                            cudaEvent_t before_check, unsigned* launches = nullptr);
-// the per-wave checker of a single trace of n records (hr_variant_runs(variant)), after the pre-pass (hr_runs.cu)
+// hr_run_kernel for a single trace of n records, after the pre-pass (hr_runs.cu)
 cudaError_t hr_launch_runs(hr_region_dev* d_regions, const hr_work& w, unsigned long long n,
                            const unsigned char* d_table, unsigned variant, cudaStream_t stream);
 // interval size and count for a job of n records when it may use up to budget intervals

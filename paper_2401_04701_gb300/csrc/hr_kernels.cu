@@ -105,6 +105,7 @@ __device__ void reset_ctl(hr_ctl* c, unsigned n_waves)
     c->bin_skip = 0;
     c->bin_err = 0;
     c->bin_every = 0;
+    c->run_items = 0;
     c->bin_tbits = 0;
     c->n_waves = n_waves;
 }
@@ -442,6 +443,11 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
     unsigned long long waves = found;
     if (w.cont) waves += rg.group_waves - (key_at(jb.trace, 0, jb.kb) == rg.last_key);  // (a wave cut in two counts once)
     const bool over = waves > w.max_waves || found > w.max_waves;
+    const bool tiled = w.check_tile && hr_waves_tiled(jb.n, found);
+    if (tiled) {
+        w.tile = w.check_tile;
+        w.clear_words = HR_CLEAR_WORDS;
+    }
     if (threadIdx.x == 0) {
         hr_jobd j0 = jb;
         j0.done_ns = 0;
@@ -466,6 +472,7 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
     }
     __syncthreads();
     stages_one_job(w, regions);
+    if (threadIdx.x == 0) w.ctl->run_items = tiled ? 0u : w.ctl->total_items;
     if (w.bin.automatic) {
         __syncthreads();
         bin_choose(w, jb, rg, s_list.at);
@@ -841,6 +848,7 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     hr_grid_wait();
+    if (w.check_tile && w.ctl->run_items) return;  // hr_run_kernel has the items
     __syncthreads();
 
     if (wid == HR_CONSUMERS) {
@@ -1266,7 +1274,9 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
     // the per-wave checker runs after it (and finds no work when binned)
     if (variant == HR_BIN_VARIANT) variant = HR_BIN_FALLBACK;
     hr_work w = w_in;
-    const bool runs = n_jobs == 1 && hr_variant_runs(variant);
+    const hr_route route = n_jobs == 1 ? hr_single_route(variant, jobs[0].n) : HR_ROUTE_TILES;
+    const bool runs = route != HR_ROUTE_TILES;
+    w.check_tile = route == HR_ROUTE_BY_WAVES ? hr_variant_tile(variant) : 0u;
     w.tile = runs ? hr_run_tile(variant) : hr_variant_tile(variant);
     w.clear_words = runs ? hr_clear_words(w.n_words, HR_RUN_CLEAR_WORDS) : HR_CLEAR_WORDS;
     w.consumers = hr_variant_consumers(variant);
@@ -1291,24 +1301,26 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
         hr_build_stages<<<1, 1024, 0, stream>>>(w, d_regions);
     }
     if (before_check) cudaEventRecord(before_check, stream);
-    if (launches) *launches = prepass_launches + 1 + (binned ? 5 : 0) + (w.tell ? 1 : 0);
+    if (launches) *launches = prepass_launches + 1 + (w.check_tile ? 1 : 0) + (binned ? 5 : 0) + (w.tell ? 1 : 0);
     if (binned) {
         const cudaError_t e = hr_launch_binned(d_regions, w, d_table, stream);
         if (e != cudaSuccess) return e;
     }
+    if (route != HR_ROUTE_RUNS) {
+        const int grid = hr_check_grid_size(variant);
+        switch (variant) {
+        case 0: launch_variant<true, 4, 8>(grid, d_regions, w, d_table, stream); break;
+        case 1: launch_variant<false, 4, 8>(grid, d_regions, w, d_table, stream); break;
+        case 2: launch_variant<true, 2, 8>(grid, d_regions, w, d_table, stream); break;
+        case 3: launch_variant<false, 2, 8>(grid, d_regions, w, d_table, stream); break;
+        case 4: launch_variant<true, 1, 8>(grid, d_regions, w, d_table, stream); break;
+        case 5: launch_variant<false, 1, 8>(grid, d_regions, w, d_table, stream); break;
+        default: launch_variant<false, 2, 8, true>(grid, d_regions, w, d_table, stream); break;
+        }
+    }
     if (runs) {
         const cudaError_t e = hr_launch_runs(d_regions, w, jobs[0].n, d_table, variant, stream);
-        return e != cudaSuccess ? e : launch_tell(d_regions, w, n_jobs, stream);
-    }
-    const int grid = hr_check_grid_size(variant);
-    switch (variant) {
-    case 0: launch_variant<true, 4, 8>(grid, d_regions, w, d_table, stream); break;
-    case 1: launch_variant<false, 4, 8>(grid, d_regions, w, d_table, stream); break;
-    case 2: launch_variant<true, 2, 8>(grid, d_regions, w, d_table, stream); break;
-    case 3: launch_variant<false, 2, 8>(grid, d_regions, w, d_table, stream); break;
-    case 4: launch_variant<true, 1, 8>(grid, d_regions, w, d_table, stream); break;
-    case 5: launch_variant<false, 1, 8>(grid, d_regions, w, d_table, stream); break;
-    default: launch_variant<false, 2, 8, true>(grid, d_regions, w, d_table, stream); break;
+        if (e != cudaSuccess) return e;
     }
     return launch_tell(d_regions, w, n_jobs, stream);
 }

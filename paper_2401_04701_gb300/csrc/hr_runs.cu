@@ -1,5 +1,5 @@
 // hr_runs.cu - the per-wave checker of single traces (sm_103a): variants 0 to 3,
-// and every-epoch regions.
+// and every-epoch regions whose waves suit it (hr_single_route()).
 //
 // Like hr_check_kernel (hr_kernels.cu) it applies the trace wave by wave to the
 // shadow in HBM, after the same pre-pass, and orders the waves with a completion
@@ -243,7 +243,7 @@ __global__ void __launch_bounds__(CHECK_THREADS, RPL >= 4 ? 2 : 3)
         for (unsigned i = threadIdx.x; i < FLIGHT; i += CHECK_THREADS) s_flight[i] = 0u;
     }
     hr_grid_wait();
-    const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->total_items;  // binned: the work is done already
+    const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->run_items;  // binned: the work is done already
     if (total == 0) return;
     // items per claim: enough to keep the ticket counter out of the way, few
     // enough that a stage's items spread over all warps
