@@ -388,6 +388,7 @@ static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_t
     w.test_flags = ctx->test_flags;
     w.views = r.views ? 1u : 0u;
     w.n_words = r.desc.n_words;
+    w.pow2 = hr_desc_geom(r.desc).bd_shift != ~0u;
     w.cont = cont ? 1u : 0u;
     w.tell = 1u;
     unsigned variant = ctx->chosen ? ctx->variant : hr_default_variant(n, r.desc.n_words);
@@ -582,6 +583,7 @@ extern "C" hr_status hr_check_batch(hr_ctx* ctx, const hr_job* jobs, uint32_t n_
     if (ctx->profile) cudaEventRecord(pc.begin, s);
     hr_work w = ctx->batch;
     w.n_words = ctx->regions[js[0].region].desc.n_words;  // (one job runs as a single trace)
+    w.pow2 = hr_desc_geom(ctx->regions[js[0].region].desc).bd_shift != ~0u;
     w.tell = 1u;
     w.wait_ns = ctx->wait_ns;
     w.cas_cap = ctx->cas_cap;

@@ -273,6 +273,7 @@ struct hr_work {
     unsigned check_tile;             // 0, or both per-wave checkers are launched: hr_check_kernel's records per item
     unsigned long long clear_words;  // shadow words per clear item (likewise)
     unsigned long long n_words;      // single traces: words of the region
+    unsigned pow2;                   // single traces: 1: block size and warp size are powers of two
     unsigned consumers;              // per-warp completions per work item
     unsigned cas_cap;                // CAS retries before HR_ERR_CONTENTION
     unsigned long long wait_ns;      // bound of every device-side wait
@@ -387,15 +388,31 @@ constexpr unsigned HR_RUN_EVERY_RPL = 4;  // records per lane in every-epoch reg
 enum hr_route { HR_ROUTE_RUNS, HR_ROUTE_TILES, HR_ROUTE_BY_WAVES };
 constexpr unsigned long long HR_EVERY_RUNS_MIN_N = 1ull << 21;  // records, and of a wave:
 constexpr unsigned long long HR_EVERY_RUNS_MIN_WAVE = 98304, HR_EVERY_RUNS_MAX_WAVE = 1250000;
-constexpr hr_route hr_single_route(unsigned v, unsigned long long n)
+// First-race regions: a single block's shared array, met again and again between
+// barriers, changes state with nearly every access, so looking for absorbed accesses
+// first only adds to them: most where a block of odd size makes every look three
+// divisions, and where lanes are aggregated.  A launch on as few words (a small graph)
+// has one wave or a few, and there hr_run_kernel is ahead by 1.1 to 1.8.  Reductions of 6
+// to 10 waves, hr_check_kernel / hr_run_kernel, variants 1, 2, 3: 0.63M records of
+// 352-thread blocks 132 / 132, 117 / 132, 91 / 103; 2.1M of 352-thread blocks 138 / 156,
+// 146 / 167, 115 / 139; 7.1M of 736-thread blocks 232 / 269, 251 / 283, 210 / 238; 10.1M of
+// 96-thread blocks 208 / 201, 269 / 222, 201 / 191; 1.06M of 256-thread blocks 115 / 104,
+// 107 / 118, 91 / 92; 10.3M of 1,024-thread blocks 238 / 263, 271 / 258, 228 / 220.
+constexpr unsigned long long HR_SMALL_WORDS = 1ull << 14;
+constexpr unsigned HR_SMALL_RUNS_WAVES = 4;  // waves that stay with hr_run_kernel
+constexpr hr_route hr_single_route(unsigned v, unsigned long long n, unsigned long long n_words, bool pow2)
 {
     if (v == HR_EVERY_EPOCH_VARIANT) return n < HR_EVERY_RUNS_MIN_N ? HR_ROUTE_TILES : HR_ROUTE_BY_WAVES;
-    return v < 4 ? HR_ROUTE_RUNS : HR_ROUTE_TILES;
+    if (v >= 4) return HR_ROUTE_TILES;
+    const bool large = n >= 1ull << 23, odd = !pow2 && n >= 1ull << 19 && !large;
+    const bool tiles = v == 1 ? odd || (pow2 && large) : v == 2 ? n >= 1ull << 18 && !large : v == 3 && odd;
+    return tiles && n_words <= HR_SMALL_WORDS ? HR_ROUTE_BY_WAVES : HR_ROUTE_RUNS;
 }
 // HR_ROUTE_BY_WAVES: whether hr_check_kernel takes a trace of n records in `waves` waves
-__host__ __device__ constexpr bool hr_waves_tiled(unsigned long long n, unsigned waves)
+__host__ __device__ constexpr bool hr_waves_tiled(bool every, unsigned long long n, unsigned waves)
 {
-    return n < waves * HR_EVERY_RUNS_MIN_WAVE || n > waves * HR_EVERY_RUNS_MAX_WAVE;
+    return every ? n < waves * HR_EVERY_RUNS_MIN_WAVE || n > waves * HR_EVERY_RUNS_MAX_WAVE
+                 : waves > HR_SMALL_RUNS_WAVES;
 }
 constexpr unsigned hr_run_tile(unsigned v)
 {

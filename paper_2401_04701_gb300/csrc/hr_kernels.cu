@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
     unsigned long long waves = found;
     if (w.cont) waves += rg.group_waves - (key_at(jb.trace, 0, jb.kb) == rg.last_key);  // (a wave cut in two counts once)
     const bool over = waves > w.max_waves || found > w.max_waves;
-    const bool tiled = w.check_tile && hr_waves_tiled(jb.n, found);
+    const bool tiled = w.check_tile && hr_waves_tiled(rg.geom.report_mode == HR_REPORT_EVERY_EPOCH, jb.n, found);
     if (tiled) {
         w.tile = w.check_tile;
         w.clear_words = HR_CLEAR_WORDS;
@@ -1274,7 +1274,7 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
     // the per-wave checker runs after it (and finds no work when binned)
     if (variant == HR_BIN_VARIANT) variant = HR_BIN_FALLBACK;
     hr_work w = w_in;
-    const hr_route route = n_jobs == 1 ? hr_single_route(variant, jobs[0].n) : HR_ROUTE_TILES;
+    const hr_route route = n_jobs == 1 ? hr_single_route(variant, jobs[0].n, w.n_words, w.pow2 != 0) : HR_ROUTE_TILES;
     const bool runs = route != HR_ROUTE_TILES;
     w.check_tile = route == HR_ROUTE_BY_WAVES ? hr_variant_tile(variant) : 0u;
     w.tile = runs ? hr_run_tile(variant) : hr_variant_tile(variant);
