@@ -498,9 +498,12 @@ __global__ void __launch_bounds__(1024) hr_batch_count(const __grid_constant__ J
     }
 }
 
-// ... then their starts and keys, after those of the jobs before.  Measured on 64
-// traces (110M records), both kernels and hr_build_stages: 105 us
-// (213 us with one scan over all jobs' intervals in four launches).
+// ... then their starts and keys, after those of the jobs before (gridDim.y CTAs a job:
+// its warps' walk over the job's intervals is a chain of look-ups, which a batch of few
+// jobs otherwise waits for).  Measured on 64 traces (110M records), both kernels and
+// hr_build_stages: 105 us (213 us with one scan over all jobs' intervals in four
+// launches) with one CTA a job; on 4 traces (9.7M records) 67 us with one, 39 with 8.
+constexpr unsigned BATCH_WAVES_CTAS = 8;  // CTAs a job, at most
 __global__ void __launch_bounds__(1024) hr_batch_waves(const __grid_constant__ JobParams<HR_MAX_BATCH> P, hr_work w)
 {
     const hr_jobd& jb = P.job[blockIdx.x];
@@ -508,7 +511,8 @@ __global__ void __launch_bounds__(1024) hr_batch_waves(const __grid_constant__ J
     block_exclusive_scan(threadIdx.x < blockIdx.x ? w.jobs[threadIdx.x].n_waves : 0u, &total);  // (blockIdx.x < 1024)
     const unsigned found = w.jobs[blockIdx.x].n_waves;
     const unsigned* counts = w.counts + jb.int_begin;
-    for (unsigned i = threadIdx.x >> 5; i < jb.n_int; i += blockDim.x >> 5) {
+    const unsigned warps = gridDim.y * (blockDim.x >> 5);
+    for (unsigned i = blockIdx.y * (blockDim.x >> 5) + (threadIdx.x >> 5); i < jb.n_int; i += warps) {
         const unsigned off = counts[i], next = i + 1 < jb.n_int ? counts[i + 1] : found;
         if (off != next) write_interval(jb, w, i, total, off);
     }
@@ -1297,7 +1301,8 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
         P.n = n_jobs;
         for (unsigned j = 0; j < n_jobs; ++j) P.job[j] = jobs[j];
         hr_batch_count<<<n_jobs, 1024, 0, stream>>>(P, w, d_regions);
-        hr_batch_waves<<<n_jobs, 1024, 0, stream>>>(P, w);
+        const unsigned parts = BATCH_WAVES_CTAS < 128 / n_jobs ? BATCH_WAVES_CTAS : 128 / n_jobs;  // one round of CTAs
+        hr_batch_waves<<<dim3(n_jobs, parts > 1 ? parts : 1), 1024, 0, stream>>>(P, w);
         hr_build_stages<<<1, 1024, 0, stream>>>(w, d_regions);
     }
     if (before_check) cudaEventRecord(before_check, stream);
