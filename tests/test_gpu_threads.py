@@ -57,3 +57,45 @@ def test_two_regions_from_two_threads(hr, variant):
             t.join()
     for i in range(2):
         assert got[i] == [(hr.HR_OK, len(want[i]), want[i])] * 4
+
+
+def test_first_checks_while_another_thread_captures(hr):
+    """A check that allocates its scratch, and one that outgrows it, queued by one thread while another
+    captures a graph in the strictest mode: the capture stays valid and the checks are right."""
+    import torch
+    traces = [trace_of(7), trace_of(8, n=6 * N)]
+    dev = [torch.from_numpy(t.view(np.uint8)).cuda() for t in traces]
+    x, other, side = torch.zeros(1000, device="cuda"), torch.cuda.Stream(), torch.cuda.Stream()
+    reg = dict(n_words=WORDS, block_dim=64)
+    with hr.Checker([reg] * 4) as ck:
+        ck.set_variant(3)
+        for i, d in enumerate(dev):
+            ck.check_trace(2 + i, d)
+        want = [hr.race_keys(ck.report(2 + i)[0]) for i in range(2)]
+    with hr.Checker([reg]) as ck:
+        torch.cuda.synchronize()
+        failed = []
+
+        def work():
+            try:
+                for d in dev:
+                    ck.reset(0, stream=other)
+                    ck.check_trace(0, d, stream=other)
+            except Exception as e:   # noqa: BLE001 (told by the main thread)
+                failed.append(e)
+
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=side, capture_error_mode="global"):
+            x.add_(1.0)
+            t = threading.Thread(target=work)
+            t.start()
+            t.join()
+        assert not failed
+        graph.replay()
+        torch.cuda.synchronize()
+        assert float(x.sum()) == 1000.0
+        races, status, n, _ = ck.report(0)
+        assert (status, n, hr.race_keys(races)) == (hr.HR_OK, len(want[1]), want[1])
+        ck.reset(0)
+        ck.check_trace(0, dev[0])
+        assert hr.race_keys(ck.report(0)[0]) == want[0]
