@@ -664,19 +664,22 @@ __device__ __forceinline__ void group_sync(unsigned id, unsigned n)
 // threads, 8.3M records: hr_bin_groups 102 -> 80 us).  wbits
 // is the wave's kernel tag, bc and wc placed where the form keeps them; mbc and
 // mwc mask the bc and wc fields; keep_w and keep_b keep the tid bits of a
-// warp's and of a block's first thread (~(warp_size - 1), ~(block_dim - 1)).
+// warp's and of a block's first thread (~(warp_size - 1), ~(block_dim - 1)).  The shifts
+// come by value: read through g in here, they cost 12 % where hub words make the steps of
+// one group the whole check (640,000 records, power-law: 895 and 1,020 us).
 template <bool POW2>
 __device__ __forceinline__ unsigned compact_step(unsigned x, unsigned tid, unsigned op, unsigned wbits, unsigned mbc,
-                                                 unsigned mwc, unsigned tidmask, const hr_geom& g, unsigned keep_w,
-                                                 unsigned keep_b, const unsigned char* tab, unsigned* raced)
+                                                 unsigned mwc, unsigned tidmask, const hr_geom& g, unsigned bd_shift,
+                                                 unsigned ws_shift, unsigned keep_w, unsigned keep_b,
+                                                 const unsigned char* tab, unsigned* raced)
 {
     const unsigned d = x ^ wbits;
     unsigned os = x >> 27;
     if (d & 0x07000000u) os = HR_STATE_INIT;  // another kernel's value (or INIT already)
     const unsigned xt = (x & tidmask) ^ tid;
     const unsigned trel = !POW2 ? hr_thread_rel(tid, x & tidmask, g)
-                        : xt == 0u ? HR_TREL_SAME : (xt >> g.bd_shift) ? HR_TREL_GRID
-                        : (xt >> g.ws_shift) ? HR_TREL_BLOCK : HR_TREL_WARP;
+                        : xt == 0u ? HR_TREL_SAME : (xt >> bd_shift) ? HR_TREL_GRID
+                        : (xt >> ws_shift) ? HR_TREL_BLOCK : HR_TREL_WARP;
     const unsigned srel = (d & mbc) ? HR_SREL_BLOCK : ((d & mwc) ? HR_SREL_WARP : HR_SREL_UNSYNC);
     const unsigned e = tab[(os << 6) | (op << 4) | (trel << 2) | srel];
     const unsigned ns = e & 31u, lvl = e >> 5;
@@ -824,8 +827,8 @@ __device__ __forceinline__ void pg_run(unsigned char* gbase, PCommon& C, const h
                     // one FSM step from a stored value to the value to store
                     auto step = [&](auto stored, unsigned* raced) -> decltype(stored) {
                         if constexpr (COMPACT)
-                            return compact_step<POW2>(stored, tid, op, wbits, mbc, mwc, tidmask, g, keep_w, keep_b, C.tab,
-                                                      raced);
+                            return compact_step<POW2>(stored, tid, op, wbits, mbc, mwc, tidmask, g, g.bd_shift, g.ws_shift,
+                                                      keep_w, keep_b, C.tab, raced);
                         else
                             return POW2 ? hr_fsm_step_pow2(stored, tid, op, bc, wc, ktag, g.bd_shift, g.ws_shift, C.tab,
                                                            raced)
