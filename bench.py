@@ -50,7 +50,8 @@ ALG_BYTES_PER_ACCESS_COMPACT = 24  # 16 B record + 4 B shadow read + 4 B shadow 
 
 
 KERNEL_SOURCES = ("paper_2401_04701_gb300/csrc/hr_kernels.cu", "paper_2401_04701_gb300/csrc/hr_runs.cu",
-                  "paper_2401_04701_gb300/csrc/hr_check.cuh", "paper_2401_04701_gb300/csrc/hr_binned.cu",
+                  "paper_2401_04701_gb300/csrc/hr_check.cuh", "paper_2401_04701_gb300/csrc/hr_launch.cuh",
+                  "paper_2401_04701_gb300/csrc/hr_binned.cu",
                   "paper_2401_04701_gb300/csrc/hr_internal.h", "include/hirace_device.cuh")
 BINNED_KERNELS = "hr_bin_count, hr_bin_scan_sums, hr_bin_scan, hr_bin_scatter, hr_bin_groups"
 
@@ -84,7 +85,7 @@ def checker_name(variant):
     from paper_2401_04701_gb300 import hirace
     if dict(hirace.variants())[variant]["binned"]:
         return "binned checker (variant %d): %s" % (variant, BINNED_KERNELS)
-    return "hr_check_kernel variant %d" % variant
+    return "per-wave checker variant %d" % variant
 
 
 def peaks():

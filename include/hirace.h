@@ -346,40 +346,47 @@ hr_status hr_destroy(hr_ctx* ctx);
 
 /*
  * Kernel variants and the autotuner (no paper counterpart; the tile schedule
- * of the checker).  Ids 0..5 are shapes of the per-wave checker: a variant
+ * of the checker). Ids 0..5 are shapes of the per-wave checker: a variant
  * fixes the consumer warps per CTA, the records each consumer lane takes per
  * tile and whether lanes on the same word are aggregated; even ids aggregate
- * and the odd id after each is the same shape without aggregation.  Until
+ * and the odd id after each is the same shape without aggregation. Until
  * hr_set_variant or hr_autotune chooses one (hr_get_variant then says 0), the
  * library picks the faster checker for each check by its size and, on the
  * device, its waves and a sample of its records; races, counts and shadows are
- * the same with every one.  Where that may be the binned one (single traces of 2^18
- * to 2^27 records on regions of at least 2^20 words), scratch of the size below is
- * allocated on first use - at most 3 GiB a context and a quarter of the free
- * memory, and never while `stream` is captured; without it the check takes a
- * per-wave shape.  Id 6 is the
- * binned checker, which hr_variant_desc reports with zero records per lane and
- * zero consumer warps: the accesses are moved into (4096-word shadow segment,
- * wave) buckets and persistent thread groups apply each segment's buckets to a
- * shared-memory copy of the segment, wave by wave.  It takes single-trace checks of regions of at
- * most 2^26 words with at most 256 waves per call; batches, and calls it cannot
- * take, run the per-wave checker of id 3.  So does a check of at least 2^22
- * accesses whose fullest segment holds more than 1/256 of them (one thread
- * group applies a segment, so a few hot words would serialise the check); that
- * decision is taken on the device after the count and scan passes.  Its first check on a region
- * allocates the region's bucket tables (4 bytes per segment for each of 256
- * waves plus about one count slice per SM) and an access buffer of 8 bytes per
- * record, so make that check before capturing calls into a CUDA graph.  Its shared-memory CAS loops are bounded by the same cap.  hr_autotune checks the given trace on `region` with
- * every variant (reset before each run, a warm-up then a timed run on
+ * the same whichever it picks. A choice stays with the context (hr_set_variant
+ * with id 0 chooses shape 0, not the library's pick again). Where that may be
+ * the binned one (single traces of 2^18 to 2^27 records on regions of at least
+ * 2^20 words), scratch of the size below is allocated on first use - at most 3
+ * GiB a context and a quarter of the free memory, and never while `stream` is
+ * captured; without it the check takes a per-wave shape. Id 6 is the binned
+ * checker, which hr_variant_desc reports with zero records per lane and zero
+ * consumer warps: the accesses are moved into (4096-word shadow segment, wave)
+ * buckets and persistent thread groups apply each segment's buckets to a
+ * shared-memory copy of the segment, wave by wave. It takes single-trace
+ * checks of regions of at most 2^26 words with at most 256 waves per call;
+ * batches, and calls it cannot take, run the per-wave checker of id 3. So does
+ * a check of at least 2^22 accesses whose fullest segment holds more than
+ * 1/256 of them (one thread group applies a segment, so a few hot words would
+ * serialise the check); that decision is taken on the device after the count
+ * and scan passes. Chosen, it differs from the others in two ways: a call that
+ * starts in a later kernel than the region's last record leaves zeros, not the
+ * older kernel's values (which read as INIT too), in the segments it writes;
+ * and of a trace with an error it reports no races, where the others report
+ * those before the error. Its first check on a region allocates the region's
+ * bucket tables (4 bytes per segment for each of 256 waves plus about one
+ * count slice per SM) and an access buffer of 8 bytes per record, so make that
+ * check before capturing calls into a CUDA graph. Its shared-memory CAS loops
+ * are bounded by the same cap. hr_autotune checks the given trace on `region`
+ * with every variant (reset before each run, a warm-up then a timed run on
  * `stream`, synchronous), keeps the fastest for this context's later checks,
  * writes it to *best and the per-variant milliseconds to ms[0..ms_cap), and
- * leaves the region reset.  A variant whose run ends with HR_ERR_CONTENTION or
+ * leaves the region reset. A variant whose run ends with HR_ERR_CONTENTION or
  * HR_ERR_TIMEOUT (a bound of that variant ran out) is skipped and gets -1 ms;
  * any other error is the trace's, and hr_autotune returns it.
- * Regions in HR_REPORT_EVERY_EPOCH mode always use checkers of their own (a
- * per-wave one, and a binned one picked as above when the region's shadow is
- * new or reset): the variant setting does not apply to them, and hr_autotune on
- * such a region returns HR_ERR_INVALID.
+ * Regions in HR_REPORT_EVERY_EPOCH mode always use checkers of their own
+ * (per-wave ones, and a binned one picked as above when the region's shadow is
+ * new or reset): the variant setting does not apply to them, and hr_autotune
+ * on such a region returns HR_ERR_INVALID.
  */
 uint32_t hr_variant_count(void);
 hr_status hr_variant_desc(uint32_t id, uint32_t* aggregate, uint32_t* records_per_lane, uint32_t* consumer_warps);

@@ -342,8 +342,8 @@ constexpr unsigned HR_N_SHAPES = sizeof(HR_VARIANTS) / sizeof(HR_VARIANTS[0]);
 constexpr unsigned HR_BIN_VARIANT = HR_N_SHAPES;
 constexpr unsigned HR_BIN_FALLBACK = 3;
 constexpr unsigned HR_N_VARIANTS = HR_N_SHAPES + 1;  // ids a caller may choose
-// Internal id of the checker that also carries the every-epoch path (shape of
-// variant 3); checks on regions in that report mode use it.
+// Internal id of the checkers that carry the every-epoch path (hr_check_kernel in
+// variant 3's shape, hr_run_kernel); checks on regions in that report mode use it.
 constexpr unsigned HR_EVERY_EPOCH_VARIANT = HR_N_VARIANTS;
 // Batches for which no variant was chosen: four records a lane without aggregation,
 // the fastest shape of every batch measured.  Variants 0, 1, 2, 3: 64 uneven
@@ -353,11 +353,11 @@ constexpr unsigned HR_BATCH_DEFAULT = 1;
 // Single traces for which none was chosen: two records a lane (variant 3) when words
 // are met again and again (the accesses mostly end early, and more warps hide more
 // latency) or the trace is small (its waves then reach more warps), else four
-// (variant 1).  Variants 0, 1, 2, 3: tree reductions of 0.1M, 1M and 10M records
-// 102, 72, 75, 53 us, 124, 94, 105, 79 us and 237, 199, 215, 182 us; power-law pushes
-// of 2.6M, 20M and 67M records 175, 173, 165, 173 us, 576, 550, 489, 475 us and
-// 1148, 1073, 953, 910 us; global-memory traces of 0.29M, 4.7M and 75M records
-// (variants 0, 1, 3) 289, 247, 218 us, 362, 331, 390 us and 2145, 1861, 2015 us.
+// (variant 1).  Calls with variants 0, 1, 2, 3: tree reductions of 0.1M, 1M and 10M
+// records 129, 104, 99, 80 us, 137, 106, 110, 92 us and 273, 219, 230, 194 us; power-law
+// pushes of 2.6M, 9.6M and 48M records 204, 209, 195, 204 us, 229, 215, 190, 181 us and
+// 961, 886, 778, 727 us; global-memory traces of 0.29M, 4.7M and 75M records
+// (variants 0, 1, 3) 285, 253, 214 us, 364, 324, 378 us and 2212, 1913, 1972 us.
 constexpr unsigned long long HR_SMALL_TRACE = 1ull << 19;
 constexpr unsigned hr_default_variant(unsigned long long n, unsigned long long n_words)
 {
