@@ -94,7 +94,8 @@ struct hr_ctx {
     bool chosen = false;               // the caller chose it; else checks may take the binned route
     std::mutex auto_lock;              // (threads may check different regions at once)
     unsigned long long auto_bytes = 0; // scratch allocated for checks that took that route by themselves
-    std::vector<void*> retired;        // buffers outgrown there (checks in flight may still use them)
+    std::mutex retire_lock;
+    std::vector<void*> retired;        // outgrown buffers that checks in flight or graphs may still use
     cudaStream_t copies = nullptr;     // non-blocking stream for report copies (never waits on user streams)
     void* batch_mem = nullptr;         // scratch of hr_check_batch (allocated on first use)
     // hr_check_trace_host: two device staging buffers, a copy stream, and events
@@ -106,10 +107,17 @@ struct hr_ctx {
     cudaEvent_t used[2] = {nullptr, nullptr};
     hr_work batch{};
     unsigned batch_jobs = 0;
+    bool batch_captured = false;       // a batch was queued inside a stream capture
     std::vector<int> batch_map;        // last hr_check_batch: caller's job -> device job (-1: empty trace)
     unsigned long long batch_waves = 0;
     std::vector<ProfiledCall> calls;   // profiled calls not read yet
     std::vector<ProfiledCall> spare;   // event triples to reuse
+
+    void retire(void* p)
+    {
+        std::lock_guard<std::mutex> lock(retire_lock);
+        retired.push_back(p);
+    }
 };
 
 static ProfiledCall take_events(hr_ctx* c)
@@ -269,11 +277,11 @@ extern "C" hr_status hr_init_with_buffers(hr_ctx** out, const hr_region_desc* re
 }
 
 // The binned checker's tables for the region's current size and an access
-// buffer of n records.  Growing them waits for the device (work in flight may
-// still use the old buffers); the first binned check of a region allocates.
-static hr_status ensure_bin(RegionHost& r, uint64_t n, cudaStream_t s)
+// buffer of n records.  Growing it waits for the device (work in flight may
+// still use the old buffer), or keeps the old one where a graph may replay into
+// it; the first binned check of a region allocates.
+static hr_status ensure_bin(hr_ctx* ctx, RegionHost& r, uint64_t n)
 {
-    (void)s;
     const unsigned n_seg = (unsigned)((r.desc.n_words + HR_BIN_SEG - 1) / HR_BIN_SEG);
     cudaError_t e = cudaSuccess;
     if (!r.bin_mem || r.bin.seg_cap < n_seg) {
@@ -301,8 +309,12 @@ static hr_status ensure_bin(RegionHost& r, uint64_t n, cudaStream_t s)
         r.bin.part_cap = part_cap;
     }
     if (r.bin.out_cap < n) {
-        if (r.bin.out) e = cudaDeviceSynchronize();
-        if (e == cudaSuccess) e = cudaFree(r.bin.out);
+        if (r.bin.out && r.captured) {
+            ctx->retire(r.bin.out);
+        } else {
+            if (r.bin.out) e = cudaDeviceSynchronize();
+            if (e == cudaSuccess) e = cudaFree(r.bin.out);
+        }
         r.bin.out = nullptr;
         r.bin.out_cap = 0;
         if (e == cudaSuccess) e = cudaMalloc(&r.bin.out, n * sizeof(uint2) + 16);
@@ -332,7 +344,7 @@ static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
         return false;
     cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
     if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone) return false;
-    if (r.bin_mem && r.bin.out_cap >= n) return ensure_bin(r, n, s) == HR_OK;
+    if (r.bin_mem && r.bin.out_cap >= n) return ensure_bin(ctx, r, n) == HR_OK;
     hr_bin shape{};
     hr_bin_shape(cap_seg, &shape);
     const uint64_t room = (n + n / 8 + 0xFFFFF) & ~0xFFFFFull;  // calls of about one size share a buffer
@@ -348,10 +360,10 @@ static bool auto_binned(hr_ctx* ctx, RegionHost& r, uint64_t n, cudaStream_t s)
     }
     cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
     if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess) return false;
-    if (r.bin.out) ctx->retired.push_back(r.bin.out);
+    if (r.bin.out) ctx->retire(r.bin.out);
     r.bin.out = nullptr;
     r.bin.out_cap = 0;
-    const bool ok = ensure_bin(r, room, s) == HR_OK;
+    const bool ok = ensure_bin(ctx, r, room) == HR_OK;
     cudaThreadExchangeStreamCaptureMode(&mode);
     if (ok) {
         ctx->auto_bytes += bytes;
@@ -398,7 +410,7 @@ static hr_status check_common(hr_ctx* ctx, uint32_t region, const hr_record* d_t
     if (variant == HR_BIN_VARIANT && (n >= (1ull << 32) || r.desc.n_words > (uint64_t)HR_BIN_MAX_SEGS * HR_BIN_SEG))
         variant = HR_BIN_FALLBACK;
     if (variant == HR_BIN_VARIANT) {
-        const hr_status bs = ensure_bin(r, n, s);
+        const hr_status bs = ensure_bin(ctx, r, n);
         if (bs != HR_OK) return bs;
         w.bin = r.bin;
     } else if (aggregate && auto_binned(ctx, r, n, s)) {
@@ -460,7 +472,7 @@ extern "C" hr_status hr_check_trace_host(hr_ctx* ctx, uint32_t region, const hr_
     }
     if (e != cudaSuccess) return cuda_status(e);
     hr_status st = HR_OK;
-    if (binned) st = ensure_bin(ctx->regions[region], room, s);  // (not grown between two pieces)
+    if (binned) st = ensure_bin(ctx, ctx->regions[region], room);  // (not grown between two pieces)
     uint64_t i = 0, m = 0;
     for (uint64_t off = 0; off < n && st == HR_OK; off += m, ++i) {
         const int b = (int)(i & 1);
@@ -519,7 +531,8 @@ extern "C" hr_status hr_batch_reserve(hr_ctx* ctx, uint32_t max_jobs, uint64_t m
         return HR_ERR_INVALID;
     if (ctx->batch_mem && ctx->batch_jobs >= max_jobs && ctx->batch_waves >= max_waves) return HR_OK;
     cudaError_t e = cudaDeviceSynchronize();
-    if (e == cudaSuccess && ctx->batch_mem) e = cudaFree(ctx->batch_mem);
+    if (ctx->batch_mem && ctx->batch_captured) ctx->retire(ctx->batch_mem);  // (a graph may replay into it)
+    else if (e == cudaSuccess && ctx->batch_mem) e = cudaFree(ctx->batch_mem);
     ctx->batch_mem = nullptr;
     const unsigned mj = max_jobs > ctx->batch_jobs ? max_jobs : ctx->batch_jobs;
     const unsigned mw = (unsigned)(max_waves > ctx->batch_waves ? max_waves : ctx->batch_waves);
@@ -602,6 +615,7 @@ extern "C" hr_status hr_check_batch(hr_ctx* ctx, const hr_job* jobs, uint32_t n_
     for (auto& d : js) {
         ctx->regions[d.region].fresh = false;
         if (e == cudaSuccess) e = mark_done(ctx->regions[d.region], s);
+        if (ctx->regions[d.region].captured) ctx->batch_captured = true;
     }
     return cuda_status(e);
 }
