@@ -1301,7 +1301,7 @@ cudaError_t hr_launch_jobs(hr_region_dev* d_regions, const hr_work& w_in, const 
         P.n = n_jobs;
         for (unsigned j = 0; j < n_jobs; ++j) P.job[j] = jobs[j];
         hr_batch_count<<<n_jobs, 1024, 0, stream>>>(P, w, d_regions);
-        const unsigned parts = BATCH_WAVES_CTAS < 128 / n_jobs ? BATCH_WAVES_CTAS : 128 / n_jobs;  // one round of CTAs
+        const unsigned parts = BATCH_WAVES_CTAS < 128 / n_jobs ? BATCH_WAVES_CTAS : 128 / n_jobs;  // at most 128 CTAs, or one a job
         hr_batch_waves<<<dim3(n_jobs, parts > 1 ? parts : 1), 1024, 0, stream>>>(P, w);
         hr_build_stages<<<1, 1024, 0, stream>>>(w, d_regions);
     }
