@@ -444,7 +444,7 @@ __global__ void __launch_bounds__(SCAN_THREADS) hr_bin_scan(hr_work w)
 // (cluster, segment) and merges the 4- or 8-byte stores.
 //
 // Bound by the cursors' atomics and by those open sectors.  Smaller clusters keep
-// more of the atomics in the CTA's own shared memory and fill more SMs (38 clusters
+// more of the atomics in the CTA's own shared memory and fill more SMs (36 clusters
 // of 4 against 15 of 8 on 152 SMs), but open more sectors: 2^14 segments x 76
 // clusters of 2 are 40 MB, more than L2 merges beside the record stream.  Time of
 // this kernel with CL = 2, 4, 8: 2^14 segments (75.2M records) 834, 547, 607 us;

@@ -145,7 +145,8 @@ struct hr_ctl {
     unsigned bin_count;    // binned checker: accesses counted into buckets
     unsigned bin_skip;     // automatic route: 1: the pre-pass left this check to the per-wave checker
     unsigned bin_every;    // 1: every-epoch region (binned only in the 4-byte working form)
-    unsigned run_items;    // total_items where hr_run_kernel has them, 0 where hr_check_kernel does
+    unsigned run_items;    // total_items, or 0 where both per-wave checkers are launched and hr_check_kernel has them
+    unsigned check_items;  // total_items, or 0 where both are and hr_run_kernel has them
     unsigned bin_err;      // automatic route: 1: the count pass met an error (the per-wave checker then
                            // does the check, and reports it)
 };
@@ -398,15 +399,17 @@ constexpr unsigned long long HR_EVERY_RUNS_MIN_WAVE = 98304, HR_EVERY_RUNS_MAX_W
 // 146 / 167, 115 / 139; 7.1M of 736-thread blocks 232 / 269, 251 / 283, 210 / 238; 10.1M of
 // 96-thread blocks 208 / 201, 269 / 222, 201 / 191; 1.06M of 256-thread blocks 115 / 104,
 // 107 / 118, 91 / 92; 10.3M of 1,024-thread blocks 238 / 263, 271 / 258, 228 / 220.
-constexpr unsigned long long HR_SMALL_WORDS = 1ull << 14;
+// Where each word is met thousands of times in all, most are absorbed again and
+// hr_run_kernel is ahead: 2.8M records of 768-thread blocks on 1,536 words 207 / 186.
+constexpr unsigned long long HR_SMALL_WORDS = 1ull << 14, HR_SMALL_MEETINGS = 1536;  // words, records a word
 constexpr unsigned HR_SMALL_RUNS_WAVES = 4;  // waves that stay with hr_run_kernel
 constexpr hr_route hr_single_route(unsigned v, unsigned long long n, unsigned long long n_words, bool pow2)
 {
     if (v == HR_EVERY_EPOCH_VARIANT) return n < HR_EVERY_RUNS_MIN_N ? HR_ROUTE_TILES : HR_ROUTE_BY_WAVES;
     if (v >= 4) return HR_ROUTE_TILES;
-    const bool large = n >= 1ull << 23, odd = !pow2 && n >= 1ull << 19 && !large;
-    const bool tiles = v == 1 ? odd || (pow2 && large) : v == 2 ? n >= 1ull << 18 && !large : v == 3 && odd;
-    return tiles && n_words <= HR_SMALL_WORDS ? HR_ROUTE_BY_WAVES : HR_ROUTE_RUNS;
+    const bool large = n >= 1ull << 23, odd = !pow2 && n >= 1ull << 19;
+    const bool tiles = v == 1 ? odd || large : v == 2 ? n >= 1ull << 18 && !large : v == 3 && odd && !large;
+    return tiles && n_words <= HR_SMALL_WORDS && n <= n_words * HR_SMALL_MEETINGS ? HR_ROUTE_BY_WAVES : HR_ROUTE_RUNS;
 }
 // HR_ROUTE_BY_WAVES: whether hr_check_kernel takes a trace of n records in `waves` waves
 __host__ __device__ constexpr bool hr_waves_tiled(bool every, unsigned long long n, unsigned waves)

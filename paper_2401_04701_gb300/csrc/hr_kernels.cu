@@ -106,6 +106,7 @@ __device__ void reset_ctl(hr_ctl* c, unsigned n_waves)
     c->bin_err = 0;
     c->bin_every = 0;
     c->run_items = 0;
+    c->check_items = 0;
     c->bin_tbits = 0;
     c->n_waves = n_waves;
 }
@@ -262,6 +263,7 @@ __device__ void stages_many_jobs(hr_work& w, hr_region_dev* regions)
         w.stages[base_s] = hr_stage{base_i, 0u, HR_STAGE_RECORDS, 0u, HR_NO_DEP, 0u, 0u, 0u};
         w.ctl->n_stages = base_s;
         w.ctl->total_items = base_i;
+        w.ctl->check_items = base_i;
     }
 }
 
@@ -472,7 +474,10 @@ __global__ void __launch_bounds__(1024) hr_prepass_single(const JobParams<1> P, 
     }
     __syncthreads();
     stages_one_job(w, regions);
-    if (threadIdx.x == 0) w.ctl->run_items = tiled ? 0u : w.ctl->total_items;
+    if (threadIdx.x == 0) {
+        w.ctl->run_items = tiled ? 0u : w.ctl->total_items;
+        w.ctl->check_items = tiled || !w.check_tile ? w.ctl->total_items : 0u;
+    }
     if (w.bin.automatic) {
         __syncthreads();
         bin_choose(w, jb, rg, s_list.at);
@@ -735,7 +740,7 @@ __device__ void producer_loop(hr_work& w, hr_region_dev* regions, uint4* s_rec, 
                               uint64_t* s_empty)
 {
     const uint64_t pol = policy_evict_first();
-    const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->total_items;  // binned: the work is done already
+    const unsigned total = hr_bin_taken(w.ctl) ? 0u : w.ctl->check_items;  // binned: the work is done already
     unsigned s = 0, s_begin = 0, s_end = 0, type = 0, dep = HR_NO_DEP, dep_need = 0, region = 0, last = 0;
     unsigned long long w_start = 0, w_end = 0, key = 0, kb = 0;
     const hr_record* trace = nullptr;
@@ -745,8 +750,9 @@ __device__ void producer_loop(hr_work& w, hr_region_dev* regions, uint4* s_rec, 
     // Tickets are claimed one batch ahead, so the claim's round trip to L2
     // overlaps the wait for a free slot instead of delaying every tile.  A
     // claimed tile only waits on stages of lower tickets, so holding one
-    // blocks nobody.
-    unsigned next = atomicAdd(&w.ctl->ticket, HR_TICKET_BATCH);
+    // blocks nobody.  (No claim where this kernel has no items: hr_run_kernel, launched
+    // after it, counts on the same tickets.)
+    unsigned next = total ? atomicAdd(&w.ctl->ticket, HR_TICKET_BATCH) : 0u;
     for (unsigned it = 0;; ++it) {
         const unsigned b = it % HR_RING;
         if (it >= HR_RING &&
@@ -852,7 +858,6 @@ __global__ void __launch_bounds__(Shape<HR_RPL, HR_CONSUMERS>::THREADS, Shape<HR
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     hr_grid_wait();
-    if (w.check_tile && w.ctl->run_items) return;  // hr_run_kernel has the items
     __syncthreads();
 
     if (wid == HR_CONSUMERS) {
