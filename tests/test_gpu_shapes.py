@@ -49,13 +49,14 @@ def test_every_epoch_shapes(hr, n, waves, kernels):
 
 
 @pytest.mark.parametrize("variant", [None, 0, 1, 2, 3])
-@pytest.mark.parametrize("n,block_dim,waves", [((1 << 19) - 1, 96, 9), (1 << 19, 96, 4), (1 << 19, 96, 5),
-                                               ((1 << 18) - 1, 64, 9), (1 << 18, 64, 9), ((1 << 23) - 1, 64, 5),
-                                               (1 << 23, 64, 5), ((1 << 23) - 1, 96, 30), (1 << 23, 96, 30)])
-def test_small_region_shapes(hr, variant, n, block_dim, waves):
+@pytest.mark.parametrize("n,block_dim,waves,words",
+                         [((1 << 19) - 1, 96, 9, 1 << 14), (1 << 19, 96, 4, 1 << 14), (1 << 19, 96, 5, 1 << 14),
+                          (1 << 19, 96, 5, (1 << 14) + 1), (512 * 1536, 96, 9, 512), (512 * 1536 + 1, 96, 9, 512),
+                          ((1 << 18) - 1, 64, 9, 1 << 14), (1 << 18, 64, 9, 1 << 14), ((1 << 23) - 1, 64, 5, 1 << 14),
+                          (1 << 23, 64, 5, 1 << 14), ((1 << 23) - 1, 96, 30, 1 << 14), (1 << 23, 96, 30, 1 << 14)])
+def test_small_region_shapes(hr, variant, n, block_dim, waves, words):
     """Regions of a shared array's size: variants 0 to 3 against variant 5, on and beside each line."""
     import torch
-    words = 1 << 14
     d = torch.from_numpy(trace_of(n % 83, n=n, words=words, waves=waves, kernels=2, threads=512).view(np.uint8)).cuda()
     shadows = [torch.zeros(words, dtype=torch.int64, device="cuda") for _ in range(2)]
     with hr.Checker([dict(n_words=words, block_dim=block_dim)] * 2, buffers=shadows) as ck:
